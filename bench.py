@@ -381,8 +381,8 @@ def _events(torch, stream):
 
 
 def run_single_small(args) -> dict:
-    """L = 128, 1000 sweeps: packed (one resident CTA for all sweeps, bound by that
-    one SM) vs plain int8 (two launches per sweep, launch-latency bound)."""
+    """L = 128, 1000 sweeps: packed (one CTA updates the lattice from acceptance masks
+    that the other SMs draw ahead) vs plain int8 (two launches per sweep, launch-latency bound)."""
     import torch
 
     from paper_1903_11714_gb300 import ising, workloads
@@ -405,7 +405,7 @@ def run_single_small(args) -> dict:
     return {"metric": "spin-flip attempts/ns, L=128 single lattice", "workload": "single_small",
             "unit": UNIT, "value": out["packed"], "plain_int8_value": out["int8"], "basis": "CUDA events",
             "config": cfg.as_dict(),
-            "note": "packed: one single-CTA launch for all sweeps; int8: 2 launches per sweep (launch-latency bound)"}
+            "note": "packed: a few launches, the random numbers of all sweeps drawn ahead of the update; int8: 2 launches per sweep (launch-latency bound)"}
 
 
 def run_batched(args, which: str) -> dict:

@@ -466,6 +466,10 @@ struct ising_s {
     double* d_mom = nullptr;    // 6 doubles
     uint64_t* d_sums = nullptr; // 11 limbs
     std::string kernel_note;    // which sweep kernel runs, and why (ising_specialized)
+    AheadLattice ahead{};       // packed, built-in kernel, L <= ahead_max_L(): the sweep with its
+    AheadPlan ahead_plan;       // random numbers drawn ahead (tiles = 0: the tiled kernel)
+    void* ahead_ws = nullptr;
+    bool ahead_refused = false; // no memory for the workspace
     const void* cubic_fixed[2] = {nullptr, nullptr};  // 3D: the colours' compiled instances
 };
 
@@ -519,6 +523,66 @@ int ensure_hist(ising_t h, int64_t need)
         if (rc) return rc;
     }
     return ISING_OK;
+}
+
+// The sweep with its random numbers drawn ahead: the lattice's plan and constants.
+int setup_ahead(ising_t h)
+{
+    const AheadPlan p = ahead_plan(h->L);
+    if (p.tiles == 0) return ISING_OK;
+    CK(ahead_configure(p));
+    h->ahead_plan = p;
+    AheadLattice& a = h->ahead;
+    a.home = h->planes;
+    a.status = h->eng.d_status;
+    a.key = h->seed;
+    a.t2 = h->desc.t2;
+    a.t4 = h->desc.t4;
+    a.all2 = h->desc.all2;
+    a.all4 = h->desc.all4;
+    a.L = (int32_t)h->L;
+    a.W = (int32_t)(h->L / 64);
+    a.words = (int32_t)(h->L * (h->L / 64));
+    a.strip = p.strip;
+    a.groups = p.groups;
+    a.rows = p.rows;
+    a.halo = p.halo;
+    a.tiles = p.tiles;
+    return ISING_OK;
+}
+
+// Whether a run of n sweeps goes that way.  The workspace (two mask buffers, for lattices of
+// several tiles two copies of the planes, the drawing tickets) is allocated by the first run
+// that needs it once the handle has been asked for 8 sweeps in all: it costs about 0.1 ms, the
+// tiled kernel's time for 8 sweeps of a lattice this size.  Before that, where memory is short
+// and on a stream that is being captured, the tiled kernel runs; the chain is the same.
+constexpr int64_t kAheadMinSweeps = 8;
+bool ahead_ready(ising_t h, int64_t n)
+{
+    const AheadPlan& p = h->ahead_plan;
+    if (p.tiles == 0) return false;
+    if (h->ahead_ws || ahead_alone(h->ahead, n)) return true;
+    if (h->ahead_refused || h->sweeps_done + n < kAheadMinSweeps) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    char* ws = nullptr;
+    if (cudaMalloc(&ws, (size_t)(2 * p.mask_bytes + p.copy_bytes + 256)) != cudaSuccess ||
+        cudaMemsetAsync(ws, 0, 256, h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(ws);
+        h->ahead_refused = true;
+        return false;
+    }
+    h->ahead_ws = ws;
+    AheadLattice& a = h->ahead;
+    a.ticket = reinterpret_cast<int*>(ws);
+    a.masks[0] = reinterpret_cast<uint2*>(ws + 256);
+    a.masks[1] = reinterpret_cast<uint2*>(ws + 256 + p.mask_bytes);
+    a.copy = reinterpret_cast<uint32_t*>(ws + 256 + 2 * p.mask_bytes);
+    return true;
 }
 
 int check_handle(ising_t h)
@@ -667,6 +731,7 @@ void destroy_handle(ising_t h)
     cudaFree(h->hist);
     cudaFree(h->d_me0);
     cudaFree(h->d_work3);
+    cudaFree(h->ahead_ws);
     cudaFree(h->d_mom);
     cudaFree(h->d_sums);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -758,8 +823,8 @@ int ising_init_ex(ising_t* out, int64_t L, double beta, uint64_t seed, int start
         // for this lattice's thresholds where the mode asks for it and it can be had
         const void* fixed = nullptr;
         const int mode = g_specialize.load();
-        if (L <= packed_resident_max_L()) {
-            h->kernel_note = "built-in: single-CTA resident kernel (L <= 256)";
+        if (L <= 256) {
+            h->kernel_note = "built-in: L <= 256";
         } else if (mode == ISING_SPECIALIZE_OFF) {
             h->kernel_note = "built-in: specialisation switched off";
         } else if (mode == ISING_SPECIALIZE_AUTO && L < kSpecializeMinL) {
@@ -779,6 +844,7 @@ int ising_init_ex(ising_t* out, int64_t L, double beta, uint64_t seed, int start
         std::vector<int32_t> ts = {0, (int32_t)lattice_tiles(L, tr, cw)};
         rc = h->eng.upload_tiles(ts, 1);
         if (!rc) rc = ensure_hist(h, 1024);
+        if (!rc && !fixed) rc = setup_ahead(h);
         if (rc) {
             destroy_handle(h);
             return rc;
@@ -911,16 +977,9 @@ int ising_sweep(ising_t h, int64_t n)
     if (n == 0) return ISING_OK;
     rc = ensure_hist(h, h->sweeps_done + n);
     if (rc) return rc;
-    if (h->kernel == ISING_PACKED && h->L <= packed_resident_max_L()) {
-        // small lattice: one CTA keeps both planes on chip for many sweeps per launch
-        LatticeDesc d = h->desc;
-        for (int64_t done = 0; done < n;) {
-            const int64_t chunk = std::min<int64_t>(n - done, 4096);
-            d.sweep = (uint32_t)(h->sweeps_done + done);
-            cudaError_t e = launch_packed_resident(d, (int)chunk, h->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
-            done += chunk;
-        }
+    if (ahead_ready(h, n)) {
+        h->ahead.hist = h->hist;
+        CK(launch_ahead_sweeps(h->ahead, h->ahead_plan.chunk, (uint32_t)h->sweeps_done, n, h->stream));
     } else if (h->kernel == ISING_PACKED) {
         rc = h->eng.run(n, 0);
         if (rc) return rc;

@@ -23,10 +23,45 @@ cudaError_t launch_packed_half_sweep(const TileTable& tt, int colour, int step, 
 // Allows launches of a fixed-threshold kernel with `smem` bytes of dynamic shared
 // memory (never less than two full stages) and gives its resident CTAs per SM.
 cudaError_t packed_fixed_configure(const void* fixed, size_t smem, int threads, int* blocks_per_sm);
-// One small lattice (L <= packed_resident_max_L()) swept nsweeps times by a single
-// CTA holding both planes in shared memory; writes hist[d.sweep .. +nsweeps).
-int packed_resident_max_L();
-cudaError_t launch_packed_resident(const LatticeDesc& d, int nsweeps, cudaStream_t s);
+// Sweeps with the random numbers drawn ahead of the update (sweep_ahead.cu), for one packed
+// lattice of side L <= ahead_max_L().  A plan's tiles = 0: no plan.
+struct AheadPlan {
+    int strip = 0;             // rows of a thread's strip
+    int groups = 0;            // strips one above the other in a tile (with its halo)
+    int rows = 0, halo = 0;    // a tile's own rows, and extra rows above and below them
+    int tiles = 0;
+    int chunk = 0;             // most sweeps of one launch
+    int64_t mask_bytes = 0;    // one buffer of acceptance masks (two are needed)
+    int64_t copy_bytes = 0;    // both copies of the planes (0: the lattice is one tile)
+};
+struct AheadLattice {
+    uint32_t* home;            // both planes, black then white
+    uint32_t* copy;            // two copies of them (lattices of several tiles)
+    uint2* masks[2];           // per half-sweep of a chunk and word: U < T_2, U < T_4
+    int* ticket;               // drawing steps taken of each buffer's chunk (two, zero between calls)
+    int64_t* hist;             // (M, E) pairs indexed by sweep number
+    int* status;               // set when a bounded wait runs out
+    uint64_t key;
+    uint32_t t2, t4, all2, all4;  // thresholds as in LatticeDesc
+    int32_t L, W, words;       // words: of one plane
+    int32_t strip, groups, rows, halo, tiles;  // the plan's
+};
+// What one launch does: update upd_n sweeps from upd_sweep on from masks buffer upd_buf, reading
+// the planes at src (-1: home, else a copy) and writing them at dst; draw the masks of gen_n
+// sweeps from gen_sweep on into buffer gen_buf; fill >= 0: copy home there first.  alone:
+// draw the update's masks in the same launch (a lattice of one tile, one CTA).
+struct AheadStep {
+    uint32_t upd_sweep, gen_sweep;
+    int32_t upd_n, upd_buf, src, dst;
+    int32_t gen_n, gen_buf, fill, alone;
+};
+int ahead_max_L();
+AheadPlan ahead_plan(int64_t L);
+cudaError_t ahead_configure(const AheadPlan& p);
+// Whether n sweeps are one launch of one CTA that draws its own masks (no workspace needed).
+bool ahead_alone(const AheadLattice& d, int64_t n);
+// Enqueues n sweeps, numbered from `sweep` on, in launches of at most `chunk` sweeps.
+cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s);
 cudaError_t launch_packed_advance(LatticeDesc* desc, const int32_t* count, int max_count, int steps,
                                   cudaStream_t s);
 // Cluster-resident sweeps (sweep_cluster.cu): lattices of one side L <= cluster_max_L()
