@@ -89,4 +89,11 @@ constexpr int64_t kCubicMaxL = 8192;
 // per-launch Philox constants hold for every word).
 __host__ __device__ inline bool cubic_q_small(int64_t L) { return (uint64_t)L * L * L <= (1ull << 35); }
 
+// Launches that follow one another on a stream (half-sweeps): the next may start while this one
+// still runs, up to the point where it needs this one's results.  grid_wait returns once
+// every earlier launch of the stream is complete and its writes are visible; a kernel
+// launched that way reads and writes nothing shared with them before it.
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 }  // namespace ising

@@ -7,6 +7,24 @@
 
 namespace ising {
 
+// Launches a kernel that starts with grid_wait() so that its start overlaps the end of the
+// stream's work before it.
+template <typename... P, typename... A>
+cudaError_t launch_following(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Launchers (return cudaError_t of the launch).  extra_tx > 0 makes every tile
 // barrier expect bytes that never arrive: only the timeout self-test uses it.
 // one != nullptr: a launch over that single lattice, whose descriptor (with the
