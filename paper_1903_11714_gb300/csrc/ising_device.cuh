@@ -92,7 +92,10 @@ __host__ __device__ inline bool cubic_q_small(int64_t L) { return (uint64_t)L * 
 // Launches that follow one another on a stream (half-sweeps): the next may start while this one
 // still runs, up to the point where it needs this one's results.  grid_wait returns once
 // every earlier launch of the stream is complete and its writes are visible; a kernel
-// launched that way reads and writes nothing shared with them before it.
+// launched that way reads and writes nothing shared with them before it.  A half-sweep of
+// a few small lattices is shorter than the gap between two dependent launches: four lattices of
+// L = 256 ... 1,024 take 9.3 us a sweep that way (13.0 without), a cube of L = 128 20 us (25
+// without); half-sweeps of half a millisecond are as fast either way.
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

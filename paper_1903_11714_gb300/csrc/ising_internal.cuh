@@ -25,6 +25,22 @@ cudaError_t launch_following(void (*kernel)(P...), dim3 grid, dim3 block, size_t
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// The same for a kernel known by its handle (compiled at run time), with its argument array.
+inline cudaError_t launch_following_c(const void* kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void** args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 // Launchers (return cudaError_t of the launch).  extra_tx > 0 makes every tile
 // barrier expect bytes that never arrive: only the timeout self-test uses it.
 // one != nullptr: a launch over that single lattice, whose descriptor (with the

@@ -126,17 +126,19 @@ cudaError_t launch_cubic_half_sweep(const CubicDesc& d, unsigned long long* work
         // the instance compiled for this lattice's thresholds (jit.cu), same parameters
         CubicDesc dd = d;
         void* args[] = {&dd, &colour, &sweep, &work};
-        return cudaLaunchKernel(fixed[colour], dim3(grid), dim3(kThreads3), args, 0, s);
+        return launch_following_c(fixed[colour], dim3(grid), dim3(kThreads3), 0, s, args);
     }
     if (G == 4 && colour == 1)
-        cubic_half_sweep_kernel<kThreads3, 4, true><<<grid, kThreads3, 0, s>>>(d, colour, sweep, work);
-    else if (G == 4)
-        cubic_half_sweep_kernel<kThreads3, 4, false><<<grid, kThreads3, 0, s>>>(d, colour, sweep, work);
-    else if (colour == 1)
-        cubic_half_sweep_kernel<kThreads3, 1, true><<<grid, kThreads3, 0, s>>>(d, colour, sweep, work);
-    else
-        cubic_half_sweep_kernel<kThreads3, 1, false><<<grid, kThreads3, 0, s>>>(d, colour, sweep, work);
-    return cudaGetLastError();
+        return launch_following(cubic_half_sweep_kernel<kThreads3, 4, true>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
+                                sweep, work);
+    if (G == 4)
+        return launch_following(cubic_half_sweep_kernel<kThreads3, 4, false>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
+                                sweep, work);
+    if (colour == 1)
+        return launch_following(cubic_half_sweep_kernel<kThreads3, 1, true>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
+                                sweep, work);
+    return launch_following(cubic_half_sweep_kernel<kThreads3, 1, false>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
+                            sweep, work);
 }
 
 cudaError_t launch_cubic_unpack(const uint32_t* black, const uint32_t* white, int8_t* lat, int64_t L, int64_t row0,

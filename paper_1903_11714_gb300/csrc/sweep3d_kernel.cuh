@@ -243,6 +243,8 @@ __global__ void __launch_bounds__(NT, 2) cubic_half_sweep_kernel(const __grid_co
     const int lane = threadIdx.x & 31;
     uint4* wq = queues + (threadIdx.x >> 5) * 2 * kQueueCap3;
     int qn = 0;  // entries in the warp's queue (the same in every lane)
+    grid_launch_next();
+    grid_wait();
     if (colour == 0 && blockIdx.x == 0 && threadIdx.x == 0) {
         // open this sweep's (M, E) slot: M = 2 * ups - N, E = 2 * anti - 3N
         const int64_t N = L * L * L;

@@ -30,21 +30,20 @@ int packed_smem_header_bytes(int threads)
 }
 
 template <int NT>
-void launch_nt(const TileTable& tt, const LatticeDesc* one, int colour, int step, int* status, int grid, size_t smem,
+cudaError_t launch_nt(const TileTable& tt, const LatticeDesc* one, int colour, int step, int* status, int grid, size_t smem,
                int stage_words, cudaStream_t s, long long wait_limit, uint32_t extra_tx, bool blocks)
 {
     if (one && one->tile_words != 0 && one->tile_words != one->W)
-        packed_half_sweep_kernel<NT, true, 1><<<grid, NT, smem, s>>>(tt, *one, colour, step, status, stage_words,
-                                                                     wait_limit, extra_tx);
-    else if (one)
-        packed_half_sweep_kernel<NT, true, 0><<<grid, NT, smem, s>>>(tt, *one, colour, step, status, stage_words,
-                                                                     wait_limit, extra_tx);
-    else if (blocks)
-        packed_half_sweep_kernel<NT, false, 2><<<grid, NT, smem, s>>>(tt, LatticeDesc{}, colour, step, status,
-                                                                      stage_words, wait_limit, extra_tx);
-    else
-        packed_half_sweep_kernel<NT, false, 0><<<grid, NT, smem, s>>>(tt, LatticeDesc{}, colour, step, status,
-                                                                      stage_words, wait_limit, extra_tx);
+        return launch_following(packed_half_sweep_kernel<NT, true, 1>, dim3(grid), dim3(NT), smem, s, tt, *one, colour,
+                                step, status, stage_words, wait_limit, extra_tx);
+    if (one)
+        return launch_following(packed_half_sweep_kernel<NT, true, 0>, dim3(grid), dim3(NT), smem, s, tt, *one, colour,
+                                step, status, stage_words, wait_limit, extra_tx);
+    if (blocks)
+        return launch_following(packed_half_sweep_kernel<NT, false, 2>, dim3(grid), dim3(NT), smem, s, tt, LatticeDesc{},
+                                colour, step, status, stage_words, wait_limit, extra_tx);
+    return launch_following(packed_half_sweep_kernel<NT, false, 0>, dim3(grid), dim3(NT), smem, s, tt, LatticeDesc{},
+                            colour, step, status, stage_words, wait_limit, extra_tx);
 }
 
 cudaError_t launch_packed_half_sweep(const TileTable& tt, int colour, int step, int* status, int grid, int threads,
@@ -59,22 +58,18 @@ cudaError_t launch_packed_half_sweep(const TileTable& tt, int colour, int step, 
         TileTable t = tt;
         LatticeDesc d = one ? *one : LatticeDesc{};
         void* args[] = {&t, &d, &colour, &step, &status, &stage_words, &wait_limit, &extra_tx};
-        return cudaLaunchKernel(fixed, dim3(grid), dim3(threads), args, smem, s);
+        return launch_following_c(fixed, dim3(grid), dim3(threads), smem, s, args);
     }
     switch (threads) {
     case 128:
-        launch_nt<128>(tt, one, colour, step, status, grid, smem, stage_words, s, wait_limit, extra_tx, blocks);
-        break;
+        return launch_nt<128>(tt, one, colour, step, status, grid, smem, stage_words, s, wait_limit, extra_tx, blocks);
     case 256:
-        launch_nt<256>(tt, one, colour, step, status, grid, smem, stage_words, s, wait_limit, extra_tx, blocks);
-        break;
+        return launch_nt<256>(tt, one, colour, step, status, grid, smem, stage_words, s, wait_limit, extra_tx, blocks);
     case 512:
-        launch_nt<512>(tt, one, colour, step, status, grid, smem, stage_words, s, wait_limit, extra_tx, blocks);
-        break;
+        return launch_nt<512>(tt, one, colour, step, status, grid, smem, stage_words, s, wait_limit, extra_tx, blocks);
     default:
         return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <int NT>

@@ -489,6 +489,18 @@ __global__ void __launch_bounds__(NT, (ONE ? (ISING_SWEEP_THREADS_PER_SM / NT > 
     uint4* queues = reinterpret_cast<uint4*>(smem_raw + 128 + ((2 * (NT / 32) * 4 + 127) / 128) * 128);
     uint32_t* stages = reinterpret_cast<uint32_t*>(queues + (NT / 32) * queue_cap(NT));
     const int tid = threadIdx.x;
+    grid_launch_next();
+    if (tid == 0) {
+        mbar_init(&bars[0], 1);
+        mbar_init(&bars[1], 1);
+        rel[0] = 0;
+        rel[1] = 0;
+        *done = 0;
+        acc[0] = 0;
+        acc[1] = 0;
+        fence_mbarrier_init();
+    }
+    grid_wait();
     const int count = ONE ? 1 : *tt.count;
     const int total = ONE ? (int)lattice_tiles(one.L, one.tile_rows, one.tile_words) : __ldg(tt.tile_start + count);
 
@@ -506,16 +518,6 @@ __global__ void __launch_bounds__(NT, (ONE ? (ISING_SWEEP_THREADS_PER_SM / NT > 
         }
     };
 
-    if (tid == 0) {
-        mbar_init(&bars[0], 1);
-        mbar_init(&bars[1], 1);
-        rel[0] = 0;
-        rel[1] = 0;
-        *done = 0;
-        acc[0] = 0;
-        acc[1] = 0;
-        fence_mbarrier_init();
-    }
     __syncthreads();  // the only CTA-wide barrier: from here on warps may run a tile apart
     if (tid == 0) {
         fill(blockIdx.x, 0);
