@@ -101,7 +101,8 @@ int ising_init(ising_t *out, int64_t L, double beta, uint64_t seed);
  * until ising_free); NULL makes the handle create and own a non-blocking stream.  Device memory: packed L*L/8
  * bytes, int8 L*L bytes, plus 16 bytes of history per sweep (grown on demand); packed
  * sides up to 8192 take a workspace for random numbers drawn ahead as well (2 to 16 MB up
- * to L = 320, 4 L^2 to 8 L^2 bytes beyond; where it cannot be had, the sweeps run without it).
+ * to L = 192, at most 16 L^2 bytes beyond, taken by the first run of 8 sweeps or more; where
+ * it cannot be had, the sweeps run without it).
  * Errors: EINVAL (L, beta, start, kernel), ENOMEM, ECUDA.
  */
 int ising_init_ex(ising_t *out, int64_t L, double beta, uint64_t seed, int start, int kernel, void *stream);

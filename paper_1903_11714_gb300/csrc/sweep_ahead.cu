@@ -45,10 +45,13 @@ constexpr int kMaxSlots = 16;
 constexpr int kMaxStrip = 16;       // rows of a thread's strip at most
 constexpr int kItemWords = 128;     // plane words of one drawing step of a warp: four a lane
 
-// Words still undecided after two Philox calls, per warp.
+// Words with sites still undecided, per warp: the next call each needs is in the entry, so that
+// a drain draws one call for 32 words that all need it.  31 may be left over when the words of a
+// pair of lanes' steps are pushed.
+constexpr int kQueueWords = 31 + 2 * 32 + 1;
 struct DrawQueue {
-    uint4 e[kItemWords];     // undecided against T_2, against T_4, below T_2 so far, below T_4
-    uint32_t at[kItemWords]; // word
+    uint4 e[kQueueWords];    // undecided against T_2, against T_4, below T_2 so far, below T_4
+    uint2 at[kQueueWords];   // word; half-sweep of the chunk << 3 | next call
 };
 
 struct SharedAhead {
@@ -58,6 +61,7 @@ struct SharedAhead {
     DrawQueue queue[kWarps];
     uint32_t planes[3][kMaxStrip * kStrips];  // the tile's spins, word of thread t's k-th row at [k * kStrips + t]:
                                               // black after even and after odd sweeps, white
+    uint4 bits[16];                   // the thresholds' bits as masks: [c] T_2's in call c's planes, [8 + c] T_4's
     uint32_t sums[2 * kMaxChunk];     // (up spins, anti-aligned bonds) of the tile's own rows after each sweep
 };
 
@@ -73,101 +77,166 @@ __device__ __forceinline__ void compare_plane(uint32_t R, uint32_t K, uint32_t& 
 
 __device__ __forceinline__ uint32_t plane_mask(uint32_t t, int plane) { return (uint32_t)((int32_t)(t << plane) >> 31); }
 
-// Draws the acceptance masks of words word0 + lane + 32 j (j < G) below `words` of one
-// half-sweep into out[word] = (U < T_2, U < T_4).  Two calls (planes 7..4, then 3..0) are drawn
-// for every word: they decide about 78 % of the words for all 32 sites and both thresholds;
-// the others finish from the warp's queue, a word per lane.
-template <int G>
-__device__ void draw_words(const AheadLattice& d, uint32_t sweep, int colour, int word0, uint2* __restrict__ out,
-                           DrawQueue& q, int lane)
+// A drawing warp's constants (one lattice) and queue.
+struct Draw {
+    uint64_t key;
+    uint32_t all2, all4;
+    const uint4* bits; // SharedAhead::bits
+    int words;
+    uint32_t sweep0;   // the chunk's first sweep
+    uint2* masks;      // of half-sweep hs at hs * words: (U < T_2, U < T_4)
+    DrawQueue* q;
+    int qn;            // entries queued (the same in every lane)
+    int lane;
+};
+
+// One call for the top n queue entries, a word per lane; words still undecided go back.
+__device__ __forceinline__ void drain_draws(Draw& w, int n)
 {
-    const PhiloxWordConsts pc = philox_consts(d.key, 0u, sweep, (uint32_t)colour);
+    const bool act = w.lane < n;
+    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    uint2 at = make_uint2(0u, 2u);
+    if (act) {
+        e = w.q->e[w.qn - n + w.lane];
+        at = w.q->at[w.qn - n + w.lane];
+    }
+    w.qn -= n;
+    __syncwarp();  // entries read before any goes back
+    const uint32_t c = at.y & 7u, hs = at.y >> 3;
+    const PhiloxWordConsts pc = philox_consts(w.key, 0u, w.sweep0 + (hs >> 1), hs & 1u);
+    const uint32_t base[1] = {8u * at.x ^ pc.x0k};
+    uint32_t o[1][4];
+    philox_calls<1>(base, c, pc, w.key, o);
+    uint32_t l2 = 0u, l4 = 0u, e2 = e.x, e4 = e.y;
+    const uint4 b2 = w.bits[c], b4 = w.bits[8 + c];
+    compare_plane(o[0][3], b2.w, l2, e2);
+    compare_plane(o[0][2], b2.z, l2, e2);
+    compare_plane(o[0][1], b2.y, l2, e2);
+    compare_plane(o[0][0], b2.x, l2, e2);
+    compare_plane(o[0][3], b4.w, l4, e4);
+    compare_plane(o[0][2], b4.z, l4, e4);
+    compare_plane(o[0][1], b4.y, l4, e4);
+    compare_plane(o[0][0], b4.x, l4, e4);
+    e.z |= e.x & l2;
+    e.w |= e.y & l4;
+    // a site still tied after all 32 planes has U equal to min(T, 2^32 - 1): below only if T = 2^32
+    if (c == 7u) {
+        e.z |= e2 & w.all2;
+        e.w |= e4 & w.all4;
+    }
+    const bool pend = (e2 | e4) != 0u && c < 7u;
+    if (act && !pend) w.masks[(size_t)hs * w.words + at.x] = make_uint2(e.z, e.w);
+    const uint32_t bal = __ballot_sync(0xffffffffu, pend);
+    if (pend) {
+        const int slot = w.qn + __popc(bal & ((1u << w.lane) - 1u));
+        w.q->e[slot] = make_uint4(e2, e4, e.z, e.w);
+        w.q->at[slot] = make_uint2(at.x, at.y + 1u);
+    }
+    w.qn += __popc(bal);
+}
+
+// Draws words word0 + lane + 32 j (j < G) of one half-sweep (FULL: all of them exist).  Two calls (planes 7..4, then 3..0)
+// for every word, side by side: they decide about 78 % of the words for all 32 sites and both
+// thresholds; the others finish from the warp's queue, a word per lane.
+template <int G, bool FULL>
+__device__ __forceinline__ void draw_words(Draw& w, const PhiloxWordConsts& pc, int hs, int word0,
+                                           const uint32_t (&K2)[8], const uint32_t (&K4)[8])
+{
     uint32_t base[G], lt2[G], lt4[G], eq2[G], eq4[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) {
-        base[j] = 8u * (uint32_t)(word0 + lane + 32 * j) ^ pc.x0k;
+        base[j] = 8u * (uint32_t)(word0 + w.lane + 32 * j) ^ pc.x0k;
         lt2[j] = lt4[j] = 0u;
         eq2[j] = eq4[j] = ~0u;
     }
 #pragma unroll
     for (int c = 1; c >= 0; --c) {
         uint32_t o[G][4];
-        philox_calls<G>(base, (uint32_t)c, pc, d.key, o);
+        philox_calls<G>(base, (uint32_t)c, pc, w.key, o);
 #pragma unroll
-        for (int m = 3; m >= 0; --m) {
-            const uint32_t K2 = plane_mask(d.t2, 4 * c + m), K4 = plane_mask(d.t4, 4 * c + m);
+        for (int m = 3; m >= 0; --m)
 #pragma unroll
             for (int j = 0; j < G; ++j) {
-                compare_plane(o[j][m], K2, lt2[j], eq2[j]);
-                compare_plane(o[j][m], K4, lt4[j], eq4[j]);
+                compare_plane(o[j][m], K2[4 * c + m], lt2[j], eq2[j]);
+                compare_plane(o[j][m], K4[4 * c + m], lt4[j], eq4[j]);
             }
-        }
     }
-    int qn = 0;
+    uint2* const out = w.masks + (size_t)hs * w.words + word0 + w.lane;
 #pragma unroll
     for (int j = 0; j < G; ++j) {
-        const int word = word0 + lane + 32 * j;
-        const bool valid = word < d.words;
-        lt2[j] |= d.all2;  // a threshold of 2^32 accepts every uniform
-        lt4[j] |= d.all4;
-        eq2[j] &= ~d.all2;
-        eq4[j] &= ~d.all4;
+        const int word = word0 + w.lane + 32 * j;
+        const bool valid = FULL || word < w.words;
         const bool pend = valid && (eq2[j] | eq4[j]) != 0u;
-        if (valid && !pend) out[word] = make_uint2(lt2[j], lt4[j]);
+        if (valid && !pend) out[32 * j] = make_uint2(lt2[j], lt4[j]);
         const uint32_t bal = __ballot_sync(0xffffffffu, pend);
         if (pend) {
-            const int slot = qn + __popc(bal & ((1u << lane) - 1u));
-            q.e[slot] = make_uint4(eq2[j], eq4[j], lt2[j], lt4[j]);
-            q.at[slot] = (uint32_t)word;
+            const int slot = w.qn + __popc(bal & ((1u << w.lane) - 1u));
+            w.q->e[slot] = make_uint4(eq2[j], eq4[j], lt2[j], lt4[j]);
+            w.q->at[slot] = make_uint2((uint32_t)word, (uint32_t)hs << 3 | 2u);
         }
-        qn += __popc(bal);
-    }
-    __syncwarp();
-    for (int first = 0; first < qn; first += 32) {
-        const bool act = first + lane < qn;
-        uint4 e = make_uint4(0u, 0u, 0u, 0u);
-        uint32_t at = 0u;
-        if (act) {
-            e = q.e[first + lane];
-            at = q.at[first + lane];
-        }
-        const uint32_t b1[1] = {8u * at ^ pc.x0k};
-        for (int c = 2; c < 8 && __any_sync(0xffffffffu, (e.x | e.y) != 0u); ++c) {
-            uint32_t o[1][4];
-            philox_calls<1>(b1, (uint32_t)c, pc, d.key, o);
-            uint32_t l2 = 0u, l4 = 0u, t2 = e.x, t4 = e.y;
-#pragma unroll
-            for (int m = 3; m >= 0; --m) {
-                compare_plane(o[0][m], plane_mask(d.t2, 4 * c + m), l2, t2);
-                compare_plane(o[0][m], plane_mask(d.t4, 4 * c + m), l4, t4);
+        w.qn += __popc(bal);
+        if ((j & 1) || j == G - 1)
+            while (w.qn >= 32) {
+                __syncwarp();  // pushes visible to the draining lanes
+                drain_draws(w, 32);
             }
-            e.z |= e.x & l2;
-            e.w |= e.y & l4;
-            e.x = t2;
-            e.y = t4;
-        }
-        // a site still tied after all 32 planes has U equal to its threshold: not below
-        if (act) out[at] = make_uint2(e.z, e.w);
     }
-    __syncwarp();  // the queue is read before the next step fills it
 }
 
-// Drawing step `item` of a chunk: steps run over the chunk's half-sweeps, each in blocks of
-// 32 G words.  The step that holds a sweep's first words also opens the sweep's (M, E) entry
-// when several tiles will add their counts to it.
-template <int G>
-__device__ __forceinline__ void draw_item(const AheadLattice& d, uint32_t sweep0, int item, uint2* masks, DrawQueue& q,
-                                          int lane)
+// The thresholds' bits as masks, for the drains; formed by one warp of the CTA.
+__device__ __forceinline__ void form_bits(const AheadLattice& d, SharedAhead& sh, int lane)
 {
-    const int per = (d.words + 32 * G - 1) / (32 * G);
-    const int hs = item / per, word0 = (item - hs * per) * 32 * G;
-    const uint32_t sweep = sweep0 + (uint32_t)(hs >> 1);
-    if (d.tiles > 1 && (hs & 1) == 0 && word0 == 0 && lane == 0) {
-        const int64_t N = (int64_t)d.L * d.L;
-        d.hist[2 * (int64_t)sweep] = -N;
-        d.hist[2 * (int64_t)sweep + 1] = -2 * N;
+    uint32_t* b = reinterpret_cast<uint32_t*>(sh.bits);
+    b[lane] = plane_mask(d.t2, lane);
+    b[32 + lane] = plane_mask(d.t4, lane);
+}
+
+// A warp's part of drawing a chunk: drawing steps of up to ITEM words of one half-sweep each,
+// `take` giving the next (in lane 0).  One at a time and only when the step in hand is done: a
+// step takes a warp about 4 us, so a warp that holds one it has not begun, or several, keeps
+// the launch waiting at its end (L = 1,024: 1.45 us a sweep taking one step ahead, 1.30 so).
+// The step that holds a sweep's first words also opens the sweep's (M, E) entry when several
+// tiles will add their counts to it.
+template <int G, int ITEM, typename Take>
+__device__ void draw_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, uint2* masks, SharedAhead& sh, int warp,
+                           int lane, Take take)
+{
+    Draw w{d.key, d.all2, d.all4, sh.bits, d.words, sweep0, masks, &sh.queue[warp], 0, lane};
+    // the thresholds' bits of the first eight planes as masks, held in registers (the opaque
+    // move keeps the compiler from forming them again for every step)
+    uint32_t K2[8], K4[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        K2[k] = plane_mask(d.t2, k);
+        K4[k] = plane_mask(d.t4, k);
+        asm volatile("mov.b32 %0, %0;" : "+r"(K2[k]));
+        asm volatile("mov.b32 %0, %0;" : "+r"(K4[k]));
     }
-    draw_words<G>(d, sweep, hs & 1, word0, masks + (size_t)hs * d.words, q, lane);
+    const int per = (d.words + ITEM - 1) / ITEM, items = 2 * sweeps * per;
+    for (;;) {
+        const int item = __shfl_sync(0xffffffffu, take(), 0);
+        if (item >= items) break;
+        const int hs = item / per, first = (item - hs * per) * ITEM;
+        const uint32_t sweep = sweep0 + (uint32_t)(hs >> 1);
+        if (d.tiles > 1 && (hs & 1) == 0 && first == 0 && lane == 0) {
+            const int64_t N = (int64_t)d.L * d.L;
+            d.hist[2 * (int64_t)sweep] = -N;
+            d.hist[2 * (int64_t)sweep + 1] = -2 * N;
+        }
+        const PhiloxWordConsts pc = philox_consts(d.key, 0u, sweep, (uint32_t)(hs & 1));
+        if (first + ITEM <= d.words) {
+#pragma unroll 1
+            for (int k = 0; k < ITEM; k += 32 * G) draw_words<G, true>(w, pc, hs, first + k, K2, K4);
+        } else {
+#pragma unroll 1
+            for (int word0 = first; word0 < d.words; word0 += 32) draw_words<1, false>(w, pc, hs, word0, K2, K4);
+        }
+    }
+    while (w.qn > 0) {
+        __syncwarp();
+        drain_draws(w, min(w.qn, 32));
+    }
+    __syncwarp();
 }
 
 // Named barriers of a tile's `threads` threads: of those that hold strips and those that count,
@@ -539,12 +608,16 @@ __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ A
     extern __shared__ __align__(16) unsigned char smem_ahead[];
     SharedAhead& sh = *reinterpret_cast<SharedAhead*>(smem_ahead);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_launch_next();
+    if (warp == 0) form_bits(d, sh, lane);
+    __syncthreads();
+    grid_wait();
     if (st.alone) {
         // a short run of a lattice of one tile: this CTA draws the masks it needs itself, into
         // the ring's slots
-        const int items = 2 * st.upd_n * ((d.words + 31) / 32);
-        for (int item = warp; item < items; item += kWarps)
-            draw_item<1>(d, st.upd_sweep, item, reinterpret_cast<uint2*>(sh.ring), sh.queue[warp], lane);
+        int next = warp - kWarps;
+        draw_chunk<1, 32>(d, st.upd_sweep, st.upd_n, reinterpret_cast<uint2*>(sh.ring), sh, warp, lane,
+                          [&] { return next += kWarps; });
         __syncthreads();
     }
     if (st.upd_n > 0)
@@ -561,23 +634,15 @@ __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ A
         d.ticket[st.gen_buf ^ 1] = 0;
         if (st.gen_n == 0) d.ticket[st.gen_buf] = 0;
     }
-    if (st.gen_n > 0) {
-        const int items = 2 * st.gen_n * ((d.words + kItemWords - 1) / kItemWords);
-        for (;;) {
-            int item = 0;
-            if (lane == 0) item = atomicAdd(&d.ticket[st.gen_buf], 1);
-            item = __shfl_sync(0xffffffffu, item, 0);
-            if (item >= items) break;
-            draw_item<4>(d, st.gen_sweep, item, d.masks[st.gen_buf], sh.queue[warp], lane);
-        }
-    }
+    if (st.gen_n > 0)
+        draw_chunk<4, kItemWords>(d, st.gen_sweep, st.gen_n, d.masks[st.gen_buf], sh, warp, lane,
+                                  [&] { return lane == 0 ? atomicAdd(&d.ticket[st.gen_buf], 1) : 0; });
 }
 
 template <int K>
 cudaError_t launch_k(const AheadLattice& d, const AheadStep& st, int grid, cudaStream_t s)
 {
-    ahead_kernel<K><<<grid, kNT, sizeof(SharedAhead), s>>>(d, st);
-    return cudaGetLastError();
+    return launch_following(ahead_kernel<K>, dim3(grid), dim3(kNT), sizeof(SharedAhead), s, d, st);
 }
 
 cudaError_t launch_step(const AheadLattice& d, const AheadStep& st, cudaStream_t s)
@@ -607,20 +672,27 @@ AheadPlan ahead_plan(int64_t L)
     const int W = (int)(L / 64);
     if (L < 64 || L % 64 || L > ahead_max_L()) return p;
     const int64_t words = L * W, per_sweep = words * 2 * (int64_t)sizeof(uint2);
-    if (L <= 320) {
-        // one tile: the whole lattice in one CTA, two, four or eight rows a thread
-        p.strip = 2;
-        while (words > (int64_t)p.strip * kStrips) p.strip *= 2;
+    if (W <= 3) {
+        // one tile: the whole lattice in one CTA, two or four rows a thread
+        p.strip = words <= 2 * kStrips ? 2 : 4;
         p.groups = (int)L / p.strip;
         p.rows = (int)L;
         p.halo = 0;
         p.tiles = 1;
         p.chunk = (int)std::min<int64_t>(kMaxChunk, (8ll << 20) / per_sweep);
     } else {
-        p.strip = L <= 1024 ? 4 : (L <= 2048 ? 8 : 16);
+        // Several tiles.  A launch costs about 4 us beyond its half-sweeps, which asks for long
+        // chunks; their halo rows are updated (and their masks fetched) by two tiles, which
+        // asks for short ones, the more so the more the drawing of the own rows' masks takes.
+        // us a sweep: L = 256: 0.59 in one tile, 0.51 with strips of 2 and chunks of 24; 320:
+        // 0.81 / 0.55 (20); 512: 1.03, 0.77, 0.69 with strips of 4 and chunks of 8, 16, 24; 1,024:
+        // 1.05 (8), 0.88 (12), strips of 8 1.08 (20); 1,344: strips of 8 1.19 (16), of 16 2.0;
+        // 2,048: strips of 8 2.16 (8), of 16 1.89 (20); 4,096: 6.95 (4), 6.63 (8), 7.06 (10);
+        // 8,192: 26.7 (2), 25.9 (3), 26.6 (4)
+        p.strip = W <= 6 ? 2 : (W <= 16 ? 4 : (W <= 28 ? 8 : 16));
         p.groups = kStrips / W;
         const int held = p.groups * p.strip;  // rows a CTA holds
-        p.chunk = std::min(16, held / 8);
+        p.chunk = W <= 28 ? std::min(32, held * 3 / 16) : (W <= 32 ? held * 5 / 32 : (W <= 64 ? held / 8 : held * 3 / 32));
         p.halo = 2 * p.chunk;
         p.rows = held - 2 * p.halo;
         p.tiles = (int)((L + p.rows - 1) / p.rows);

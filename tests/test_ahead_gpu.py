@@ -32,8 +32,8 @@ def check(lat, L, beta, seed, start, runs):
     assert np.array_equal(lat.get_lattice(), ref)
 
 
-# one tile: strips of 2 rows (L = 64 ... 256) and of 4 (L = 320); several tiles beyond, with
-# rows of an even, odd and prime number of words
+# one tile: strips of 2 rows (L = 64, 128) and of 4 (192); several tiles beyond, with strips of
+# 2, 4 and 8 rows and rows of an even, odd and prime number of words
 @pytest.mark.parametrize("L", [64, 128, 192, 256, 320, 384, 448, 512, 1088])
 @pytest.mark.parametrize("beta", [0.0, 0.4406868, 200.0])
 def test_ahead_matches_oracle(L, beta):
@@ -43,7 +43,7 @@ def test_ahead_matches_oracle(L, beta):
 
 
 def test_long_runs_cross_chunks():
-    # L = 128: chunks of 64, 1024 and the rest; L = 256: chunks of at most 512
+    # L = 128: chunks of 64, 1024 and the rest; L = 256: chunks of 24
     for L, runs in ((128, [3, 1200, 40]), (256, [600, 9])):
         lat = ising.Lattice(L, 0.44, 5, ising.COLD)
         check(lat, L, 0.44, 5, ising.COLD, runs)
