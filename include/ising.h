@@ -101,7 +101,7 @@ int ising_init(ising_t *out, int64_t L, double beta, uint64_t seed);
  * until ising_free); NULL makes the handle create and own a non-blocking stream.  Device memory: packed L*L/8
  * bytes, int8 L*L bytes, plus 16 bytes of history per sweep (grown on demand); packed
  * sides up to 8192 take a workspace for random numbers drawn ahead as well (2 to 16 MB up
- * to L = 192, at most 16 L^2 bytes beyond, taken by the first run of 8 sweeps or more; where
+ * to L = 192, at most 16 L^2 bytes beyond, taken by the first run that reaches 16 sweeps; where
  * it cannot be had, the sweeps run without it).
  * Errors: EINVAL (L, beta, start, kernel), ENOMEM, ECUDA.
  */
@@ -240,8 +240,14 @@ int ising_batch_specialized(ising_batch_t b, int32_t *specialized);
  * per SM its CTAs occupy) beats the tiled kernel's (about 25.7 sites/ns per SM,
  * halved at 5e7 sites per sweep): many small lattices, or a few of L <= 2048;
  * ISING_CLUSTER_ALWAYS whenever the lattices fit.
- * ising_batch_cluster_size gives the C in use (0: the tiled kernel).  Host-only;
+ * ising_batch_cluster_size gives the C of that choice (0: the tiled kernel).  Host-only;
  * the mode is re-applied whenever lattices are added or removed.
+ * In the automatic mode a batch of sides up to 4,096 (whole-row tiles, several
+ * temperatures) and up to about 1e8 sites is swept with its random numbers drawn ahead
+ * of the update instead where that is estimated to be faster (any mix of sides; most
+ * batches of up to 5e7 sites): from its 16th sweep on, in a device workspace beside the
+ * arena of about 4 bytes a site, taken by the first such run; where it cannot be had,
+ * the other two forms run.  The chain is the same, bit for bit.
  * Paper: Sec. 3.1 (the schedule), Sec. 4.1 (scans of small lattices).
  * Errors: EINVAL (null argument, mode not 0-2).
  */

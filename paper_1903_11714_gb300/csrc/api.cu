@@ -487,6 +487,15 @@ struct ising_batch_s {
     // allocated apart from the arena and doubled when a run needs more room
     bool growable = false;
     int cluster_mode = ISING_CLUSTER_AUTO;  // ising_batch_set_cluster
+    // the sweep with its random numbers drawn ahead (update_ahead): whether it is chosen, its
+    // launch parameters, its workspace (and those it has outgrown, still in use by earlier
+    // launches), and whether its tables follow the slots
+    bool ahead_wanted = false, ahead_refused = false, ahead_tables = false;
+    AheadBatch ahead{};
+    int64_t ahead_steps = 0, ahead_asked = 0;
+    char* ahead_ws = nullptr;
+    int64_t ahead_ws_bytes = 0;
+    std::vector<void*> ahead_outgrown;
     int capacity = 0;
     int64_t max_L = 0;
     cudaStream_t stream = nullptr;
@@ -553,10 +562,10 @@ int setup_ahead(ising_t h)
 
 // Whether a run of n sweeps goes that way.  The workspace (two mask buffers, for lattices of
 // several tiles two copies of the planes, the drawing tickets) is allocated by the first run
-// that needs it once the handle has been asked for 8 sweeps in all: it costs about 0.1 ms, the
-// tiled kernel's time for 8 sweeps of a lattice this size.  Before that, where memory is short
+// that needs it once the handle has been asked for 16 sweeps in all: it costs about 0.1 ms, the
+// tiled kernel's time for 10 sweeps of a lattice this size.  Before that, where memory is short
 // and on a stream that is being captured, the tiled kernel runs; the chain is the same.
-constexpr int64_t kAheadMinSweeps = 8;
+constexpr int64_t kAheadMinSweeps = 16;
 bool ahead_ready(ising_t h, int64_t n)
 {
     const AheadPlan& p = h->ahead_plan;
@@ -1349,6 +1358,110 @@ int update_cluster(ising_batch_t b)
     return ISING_OK;
 }
 
+// A batch of few sites per sweep, whose half-sweeps the tiled kernel cannot spread over the GPU
+// for long enough to hide a launch, is swept with its random numbers drawn ahead of the update
+// (sweep_ahead.cu) instead: in the automatic mode, for sides up to 4,096 with whole-row tiles,
+// unless it sweeps with the kernel compiled for its one temperature, when the estimate is
+// the shortest.  Estimates for S sites, in ns a sweep (each a fit to measured batches):
+//  - drawn ahead: 350 + S / 2,300 (16 x 512 2.4 us, 24 x 1,280 16.9, 64 x 1,024 29.0);
+//  - tiled kernel: (S + 2.5e7) / 2,690, its rate with tall tiles (8 x 4,096: 59 us either way;
+//    32 uneven lattices of 2.1e7 sites 21.4 us, 9.5 drawn ahead); they cross at 1.2e8 sites;
+//  - cluster-resident: 3,000 + 1,420 for each word a thread holds of a plane (64 x 1,024: 16
+//    words, 25.7 us; 8 x 1,024: 8.7, drawn ahead 3.7; 256 x 128: 4.9 and 2.6).
+void update_ahead(ising_batch_t b)
+{
+    b->ahead_wanted = false;
+    b->ahead_tables = false;
+    if (b->cluster_mode != ISING_CLUSTER_AUTO || b->eng.fixed_multi || b->count < 1 || b->count > ahead_batch_max_count())
+        return;
+    int64_t sites = 0, longest = 0;
+    for (const auto& s : b->slots) {
+        if (!s.used) continue;
+        if (s.L > ahead_batch_max_L() || s.desc.tile_words != s.desc.W) return;
+        sites += s.L * s.L;
+        longest = std::max(longest, s.L);
+    }
+    if (longest == 0) return;
+    const double sms = sm_count(), S = (double)sites, drawn_ahead = 350.0 + S / (2300.0 * sms / 152.0);
+    double other = (S + 2.5e7) / (2690.0 * sms / 152.0);
+    const ClusterPlan& c = b->eng.cluster;
+    if (c.C > 0) {
+        const double plane = (double)longest * (longest / 64);
+        other = 3000.0 + 1420.0 * std::max(plane / ((double)c.C * c.threads), b->count * plane / (sms * 512.0));
+    }
+    if (drawn_ahead >= other) return;
+    b->ahead_wanted = true;
+    b->ahead.chunk = ahead_batch_chunk(longest);
+    // tall tiles once a launch has work for every SM (us a sweep, low / tall tiles: 8 x 256
+    // 0.75 / 1.08; 32 x 256 1.53 / 1.23; 16 x 512 2.40 / 2.36; 64 x 1,024 32.2 / 29.0)
+    b->ahead.dense = S >= 2e6;
+}
+
+// Whether a run of n sweeps goes that way: the workspace and the tables are made ready by the
+// first run that needs them, once the batch has been asked for 16 sweeps in all (before
+// that, where memory is short and on a stream that is being captured: the tiled or the
+// cluster-resident kernel, as otherwise).
+constexpr int64_t kAheadMinBatchSweeps = 16;
+int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
+{
+    *ready = false;
+    b->ahead_asked = std::min<int64_t>(b->ahead_asked + n, kAheadMinBatchSweeps);
+    if (!b->ahead_wanted || b->ahead_refused || b->ahead_asked < kAheadMinBatchSweeps) return ISING_OK;
+    if (b->ahead_tables) {
+        *ready = true;
+        return ISING_OK;
+    }
+    AheadBatch& a = b->ahead;
+    std::vector<int32_t> t(3 * ((size_t)b->count + 1), 0);
+    int32_t *tiles = t.data(), *steps = tiles + b->count + 1, *words = steps + b->count + 1;
+    for (int k = 0; k < b->count; ++k) {
+        const auto& s = b->slots[k];
+        tiles[k + 1] = tiles[k] + (s.used ? ahead_batch_tiles(s.L, a.chunk, a.dense) : 0);
+        steps[k + 1] = steps[k] + (s.used ? ahead_batch_steps(s.L) : 0);
+        words[k + 1] = words[k] + (s.used ? (int32_t)(s.L * (s.L / 64)) : 0);
+    }
+    const int64_t W = words[b->count], table_bytes = 256 + (3 * ((int64_t)ahead_batch_max_count() + 1) * 4 + 255) / 256 * 256;
+    const int64_t mask_bytes = (W * 2 * a.chunk * (int64_t)sizeof(uint2) + 255) / 256 * 256;
+    const int64_t need = table_bytes + 2 * mask_bytes + W * 16;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return ISING_OK;
+    }
+    if (need > b->ahead_ws_bytes) {
+        CK(ahead_batch_configure());
+        // half as much again for lattices yet to come; the outgrown workspace stays until the
+        // batch is freed, as earlier launches may still use it (all of them together are at
+        // most twice the last one)
+        char* ws = nullptr;
+        const int64_t bytes = b->ahead_ws ? need + need / 2 : need;
+        if (cudaMalloc(&ws, (size_t)bytes) != cudaSuccess) {
+            cudaGetLastError();
+            b->ahead_refused = true;
+            return ISING_OK;
+        }
+        if (b->ahead_ws) b->ahead_outgrown.push_back(b->ahead_ws);
+        b->ahead_ws = ws;
+        b->ahead_ws_bytes = bytes;
+        CK(cudaMemsetAsync(ws, 0, 256, b->stream));
+    }
+    char* ws = b->ahead_ws;
+    a.desc = b->eng.d_desc;
+    a.ticket = reinterpret_cast<int*>(ws);
+    a.tables = reinterpret_cast<const int32_t*>(ws + 256);
+    a.masks[0] = reinterpret_cast<uint2*>(ws + table_bytes);
+    a.masks[1] = reinterpret_cast<uint2*>(ws + table_bytes + mask_bytes);
+    a.copy = reinterpret_cast<uint32_t*>(ws + table_bytes + 2 * mask_bytes);
+    a.status = b->eng.d_status;
+    a.count = b->count;
+    a.tiles = tiles[b->count];
+    b->ahead_steps = steps[b->count];
+    CK(launch_set_tiles(reinterpret_cast<int32_t*>(ws + 256), nullptr, t.data(), (int32_t)t.size(), -1, b->stream));
+    b->ahead_tables = true;
+    *ready = true;
+    return ISING_OK;
+}
+
 int rebuild_tiles(ising_batch_t b)
 {
     int32_t count = 0;
@@ -1363,6 +1476,7 @@ int rebuild_tiles(ising_batch_t b)
     int rc = b->eng.upload_tiles(ts, count);
     if (!rc) rc = update_specialisation(b);
     if (!rc) rc = update_cluster(b);
+    if (!rc) update_ahead(b);
     return rc;
 }
 
@@ -1632,8 +1746,21 @@ int ising_batch_run(ising_batch_t b, int64_t sweeps, int32_t graph_sweeps)
         int rc = grow_histories(b, sweeps);
         if (rc) return rc;
     }
-    int rc = b->eng.run(sweeps, graph_sweeps);
+    bool ahead = false;
+    int rc = sweeps > 0 ? ahead_ready(b, sweeps, &ahead) : ISING_OK;
     if (rc) return rc;
+    if (ahead) {
+        // in parts whose sweep numbers fit the launch parameters; no graph is needed
+        for (int64_t done = 0; done < sweeps;) {
+            const int64_t n = std::min<int64_t>(sweeps - done, 1 << 20);
+            CK(launch_ahead_batch(b->ahead, b->ahead_steps, n, b->stream));
+            CK(launch_packed_advance(b->eng.d_desc, b->eng.d_count, b->eng.max_count, (int)n, b->stream));
+            done += n;
+        }
+    } else {
+        rc = b->eng.run(sweeps, graph_sweeps);
+        if (rc) return rc;
+    }
     if (b->growable)
         for (auto& s : b->slots)
             if (s.used) s.done += sweeps;
@@ -1666,7 +1793,9 @@ int ising_batch_set_cluster(ising_batch_t b, int32_t mode)
     if (mode != ISING_CLUSTER_OFF && mode != ISING_CLUSTER_AUTO && mode != ISING_CLUSTER_ALWAYS)
         return fail(ISING_EINVAL, "cluster mode %d is not 0, 1 or 2", mode);
     b->cluster_mode = mode;
-    return update_cluster(b);
+    const int rc = update_cluster(b);
+    if (!rc) update_ahead(b);
+    return rc;
 }
 
 int ising_batch_cluster_size(ising_batch_t b, int32_t* cluster_size)
@@ -1801,6 +1930,8 @@ int ising_batch_free(ising_batch_t b)
     b->eng.destroy();
     b->arena.destroy();
     for (auto& s : b->slots) cudaFree(s.own_hist);
+    cudaFree(b->ahead_ws);
+    for (void* p : b->ahead_outgrown) cudaFree(p);
     cudaFree(b->d_me);
     cudaFree(b->d_mom);
     cudaFree(b->d_sums);

@@ -89,6 +89,32 @@ struct AheadStep {
     int32_t upd_n, upd_buf, src, dst;
     int32_t gen_n, gen_buf, fill, alone;
 };
+// The same for the lattices of a batch (sides up to ahead_batch_max_L(), at most
+// ahead_batch_max_count() slots): every lattice's masks, copies and tiles in common launches.
+struct AheadBatch {
+    const LatticeDesc* desc;   // count slots
+    const int32_t* tables;     // prefix sums over the slots, count + 1 entries each: tiles, drawing
+                               // steps of a half-sweep, plane words
+    uint2* masks[2];           // each 2 * chunk uint2 for every plane word
+    uint32_t* copy;            // four words for every plane word
+    int* ticket;               // two, zero between runs
+    int* status;
+    int32_t count, chunk, tiles;
+    int32_t dense;             // work for every SM: tall tiles
+};
+struct AheadBatchStep {
+    int32_t total;             // sweeps of the run; a lattice stops at its own limit
+    int32_t upd_off, upd_n, upd_buf, src;
+    int32_t gen_off, gen_n, gen_buf, fill;
+};
+int ahead_batch_max_L();
+int ahead_batch_max_count();
+int ahead_batch_chunk(int64_t L);               // sweeps of a launch, for the batch's longest side
+int32_t ahead_batch_tiles(int64_t L, int chunk, int dense);
+int32_t ahead_batch_steps(int64_t L);
+cudaError_t ahead_batch_configure();
+// Enqueues a run of n sweeps; steps: drawing steps of a half-sweep of all lattices.
+cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s);
 int ahead_max_L();
 AheadPlan ahead_plan(int64_t L);
 cudaError_t ahead_configure(const AheadPlan& p);

@@ -42,6 +42,7 @@ constexpr int kWarps = kNT / 32;
 constexpr int kMaxChunk = 1024;     // sweeps per launch (their counts are kept in shared memory)
 constexpr int kRingBytes = 128 * 1024;  // masks of the coming half-sweeps, staged in shared memory
 constexpr int kMaxSlots = 16;
+constexpr int kMaxBatchChunk = 32;
 constexpr int kMaxStrip = 16;       // rows of a thread's strip at most
 constexpr int kItemWords = 128;     // plane words of one drawing step of a warp: four a lane
 
@@ -51,8 +52,10 @@ constexpr int kItemWords = 128;     // plane words of one drawing step of a warp
 constexpr int kQueueWords = 31 + 2 * 32 + 1;
 struct DrawQueue {
     uint4 e[kQueueWords];    // undecided against T_2, against T_4, below T_2 so far, below T_4
-    uint2 at[kQueueWords];   // word; half-sweep of the chunk << 3 | next call
+    uint2 at[kQueueWords];   // lattice << kWordBits | word; half-sweep of the chunk << 3 | next call
 };
+constexpr int kWordBits = 20;  // a plane has at most 2^20 words (L = 8,192)
+constexpr uint32_t kWordMask = (1u << kWordBits) - 1u;
 
 struct SharedAhead {
     alignas(128) unsigned char ring[kRingBytes];
@@ -61,7 +64,13 @@ struct SharedAhead {
     DrawQueue queue[kWarps];
     uint32_t planes[3][kMaxStrip * kStrips];  // the tile's spins, word of thread t's k-th row at [k * kStrips + t]:
                                               // black after even and after odd sweeps, white
-    uint4 bits[16];                   // the thresholds' bits as masks: [c] T_2's in call c's planes, [8 + c] T_4's
+    union {
+        uint4 bits[16];               // the thresholds' bits as masks: [c] T_2's in call c's planes, [8 + c] T_4's
+        struct {                      // batches: the tile's lattice and what to do with it
+            AheadLattice lattice;
+            AheadStep step;
+        } now;
+    };
     uint32_t sums[2 * kMaxChunk];     // (up spins, anti-aligned bonds) of the tile's own rows after each sweep
 };
 
@@ -77,21 +86,26 @@ __device__ __forceinline__ void compare_plane(uint32_t R, uint32_t K, uint32_t& 
 
 __device__ __forceinline__ uint32_t plane_mask(uint32_t t, int plane) { return (uint32_t)((int32_t)(t << plane) >> 31); }
 
-// A drawing warp's constants (one lattice) and queue.
-struct Draw {
+// What drawing needs of a lattice.
+struct DrawLattice {
     uint64_t key;
-    uint32_t all2, all4;
-    const uint4* bits; // SharedAhead::bits
+    uint32_t t2, t4, all2, all4;
     int words;
     uint32_t sweep0;   // the chunk's first sweep
     uint2* masks;      // of half-sweep hs at hs * words: (U < T_2, U < T_4)
+};
+
+// A drawing warp's queue.
+struct DrawState {
     DrawQueue* q;
     int qn;            // entries queued (the same in every lane)
     int lane;
 };
 
 // One call for the top n queue entries, a word per lane; words still undecided go back.
-__device__ __forceinline__ void drain_draws(Draw& w, int n)
+// `lattice` gives an entry's lattice, `bits` the thresholds' bits of a call's four planes.
+template <typename Lattice, typename Bits>
+__device__ __forceinline__ void drain_draws(DrawState& w, int n, Lattice lattice, Bits bits)
 {
     const bool act = w.lane < n;
     uint4 e = make_uint4(0u, 0u, 0u, 0u);
@@ -102,13 +116,15 @@ __device__ __forceinline__ void drain_draws(Draw& w, int n)
     }
     w.qn -= n;
     __syncwarp();  // entries read before any goes back
-    const uint32_t c = at.y & 7u, hs = at.y >> 3;
-    const PhiloxWordConsts pc = philox_consts(w.key, 0u, w.sweep0 + (hs >> 1), hs & 1u);
-    const uint32_t base[1] = {8u * at.x ^ pc.x0k};
+    const uint32_t word = at.x & kWordMask, c = at.y & 7u, hs = at.y >> 3;
+    const DrawLattice d = lattice((int)(at.x >> kWordBits));
+    const PhiloxWordConsts pc = philox_consts(d.key, 0u, d.sweep0 + (hs >> 1), hs & 1u);
+    const uint32_t base[1] = {8u * word ^ pc.x0k};
     uint32_t o[1][4];
-    philox_calls<1>(base, c, pc, w.key, o);
+    philox_calls<1>(base, c, pc, d.key, o);
     uint32_t l2 = 0u, l4 = 0u, e2 = e.x, e4 = e.y;
-    const uint4 b2 = w.bits[c], b4 = w.bits[8 + c];
+    uint4 b2, b4;
+    bits(d, c, b2, b4);
     compare_plane(o[0][3], b2.w, l2, e2);
     compare_plane(o[0][2], b2.z, l2, e2);
     compare_plane(o[0][1], b2.y, l2, e2);
@@ -121,11 +137,11 @@ __device__ __forceinline__ void drain_draws(Draw& w, int n)
     e.w |= e.y & l4;
     // a site still tied after all 32 planes has U equal to min(T, 2^32 - 1): below only if T = 2^32
     if (c == 7u) {
-        e.z |= e2 & w.all2;
-        e.w |= e4 & w.all4;
+        e.z |= e2 & d.all2;
+        e.w |= e4 & d.all4;
     }
     const bool pend = (e2 | e4) != 0u && c < 7u;
-    if (act && !pend) w.masks[(size_t)hs * w.words + at.x] = make_uint2(e.z, e.w);
+    if (act && !pend) d.masks[(size_t)hs * d.words + word] = make_uint2(e.z, e.w);
     const uint32_t bal = __ballot_sync(0xffffffffu, pend);
     if (pend) {
         const int slot = w.qn + __popc(bal & ((1u << w.lane) - 1u));
@@ -135,12 +151,14 @@ __device__ __forceinline__ void drain_draws(Draw& w, int n)
     w.qn += __popc(bal);
 }
 
-// Draws words word0 + lane + 32 j (j < G) of one half-sweep (FULL: all of them exist).  Two calls (planes 7..4, then 3..0)
-// for every word, side by side: they decide about 78 % of the words for all 32 sites and both
-// thresholds; the others finish from the warp's queue, a word per lane.
-template <int G, bool FULL>
-__device__ __forceinline__ void draw_words(Draw& w, const PhiloxWordConsts& pc, int hs, int word0,
-                                           const uint32_t (&K2)[8], const uint32_t (&K4)[8])
+// Draws words word0 + lane + 32 j (j < G) of one half-sweep (FULL: all of them exist).  Two
+// calls (planes 7..4, then 3..0) for every word, side by side: they decide about 78 % of the
+// words for all 32 sites and both thresholds; the others finish from the warp's queue, a word per
+// lane.  K2, K4: the thresholds' bits of the first eight planes as masks.
+template <int G, bool FULL, typename Lattice, typename Bits>
+__device__ __forceinline__ void draw_words(DrawState& w, const DrawLattice& d, int index, const PhiloxWordConsts& pc, int hs,
+                                           int word0, const uint32_t (&K2)[8], const uint32_t (&K4)[8], Lattice lattice,
+                                           Bits bits)
 {
     uint32_t base[G], lt2[G], lt4[G], eq2[G], eq4[G];
 #pragma unroll
@@ -152,7 +170,7 @@ __device__ __forceinline__ void draw_words(Draw& w, const PhiloxWordConsts& pc, 
 #pragma unroll
     for (int c = 1; c >= 0; --c) {
         uint32_t o[G][4];
-        philox_calls<G>(base, (uint32_t)c, pc, w.key, o);
+        philox_calls<G>(base, (uint32_t)c, pc, d.key, o);
 #pragma unroll
         for (int m = 3; m >= 0; --m)
 #pragma unroll
@@ -161,26 +179,50 @@ __device__ __forceinline__ void draw_words(Draw& w, const PhiloxWordConsts& pc, 
                 compare_plane(o[j][m], K4[4 * c + m], lt4[j], eq4[j]);
             }
     }
-    uint2* const out = w.masks + (size_t)hs * w.words + word0 + w.lane;
+    uint2* const out = d.masks + (size_t)hs * d.words + word0 + w.lane;
 #pragma unroll
     for (int j = 0; j < G; ++j) {
         const int word = word0 + w.lane + 32 * j;
-        const bool valid = FULL || word < w.words;
+        const bool valid = FULL || word < d.words;
         const bool pend = valid && (eq2[j] | eq4[j]) != 0u;
         if (valid && !pend) out[32 * j] = make_uint2(lt2[j], lt4[j]);
         const uint32_t bal = __ballot_sync(0xffffffffu, pend);
         if (pend) {
             const int slot = w.qn + __popc(bal & ((1u << w.lane) - 1u));
             w.q->e[slot] = make_uint4(eq2[j], eq4[j], lt2[j], lt4[j]);
-            w.q->at[slot] = make_uint2((uint32_t)word, (uint32_t)hs << 3 | 2u);
+            w.q->at[slot] = make_uint2((uint32_t)index << kWordBits | (uint32_t)word, (uint32_t)hs << 3 | 2u);
         }
         w.qn += __popc(bal);
         if ((j & 1) || j == G - 1)
             while (w.qn >= 32) {
                 __syncwarp();  // pushes visible to the draining lanes
-                drain_draws(w, 32);
+                drain_draws(w, 32, lattice, bits);
             }
     }
+}
+
+// One drawing step: words first .. first + ITEM - 1 (as far as they exist) of half-sweep hs.
+template <int G, int ITEM, typename Lattice, typename Bits>
+__device__ __forceinline__ void draw_step(DrawState& w, const DrawLattice& d, int index, int hs, int first,
+                                          const uint32_t (&K2)[8], const uint32_t (&K4)[8], Lattice lattice, Bits bits)
+{
+    const PhiloxWordConsts pc = philox_consts(d.key, 0u, d.sweep0 + (uint32_t)(hs >> 1), (uint32_t)(hs & 1));
+    if (first + ITEM <= d.words) {
+#pragma unroll 1
+        for (int k = 0; k < ITEM; k += 32 * G)
+            draw_words<G, true>(w, d, index, pc, hs, first + k, K2, K4, lattice, bits);
+    } else {
+#pragma unroll 1
+        for (int word0 = first; word0 < d.words; word0 += 32)
+            draw_words<1, false>(w, d, index, pc, hs, word0, K2, K4, lattice, bits);
+    }
+}
+
+// Opens the (M, E) entry of a sweep of an L x L lattice to which several tiles will add their counts.
+__device__ __forceinline__ void open_entry(int64_t* hist, uint32_t sweep, int64_t L)
+{
+    hist[2 * (int64_t)sweep] = -L * L;
+    hist[2 * (int64_t)sweep + 1] = -2 * L * L;
 }
 
 // The thresholds' bits as masks, for the drains; formed by one warp of the CTA.
@@ -191,19 +233,24 @@ __device__ __forceinline__ void form_bits(const AheadLattice& d, SharedAhead& sh
     b[32 + lane] = plane_mask(d.t4, lane);
 }
 
-// A warp's part of drawing a chunk: drawing steps of up to ITEM words of one half-sweep each,
-// `take` giving the next (in lane 0).  One at a time and only when the step in hand is done: a
-// step takes a warp about 4 us, so a warp that holds one it has not begun, or several, keeps
-// the launch waiting at its end (L = 1,024: 1.45 us a sweep taking one step ahead, 1.30 so).
-// The step that holds a sweep's first words also opens the sweep's (M, E) entry when several
-// tiles will add their counts to it.
+// A warp's part of drawing a chunk of one lattice: drawing steps of up to ITEM words of one
+// half-sweep each, `take` giving the next (in lane 0).  One at a time and only when the step in
+// hand is done: a step takes a warp about 4 us, so a warp that holds one it has not begun, or
+// several, keeps the launch waiting at its end (L = 1,024: 1.45 us a sweep taking one step
+// ahead, 1.30 so).  The step that holds a sweep's first words also opens the sweep's (M, E)
+// entry when several tiles will add their counts to it.
 template <int G, int ITEM, typename Take>
 __device__ void draw_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, uint2* masks, SharedAhead& sh, int warp,
                            int lane, Take take)
 {
-    Draw w{d.key, d.all2, d.all4, sh.bits, d.words, sweep0, masks, &sh.queue[warp], 0, lane};
-    // the thresholds' bits of the first eight planes as masks, held in registers (the opaque
-    // move keeps the compiler from forming them again for every step)
+    DrawState w{&sh.queue[warp], 0, lane};
+    const DrawLattice one{d.key, d.t2, d.t4, d.all2, d.all4, d.words, sweep0, masks};
+    auto lattice = [&](int) { return one; };
+    auto bits = [&](const DrawLattice&, uint32_t c, uint4& b2, uint4& b4) {
+        b2 = sh.bits[c];
+        b4 = sh.bits[8 + c];
+    };
+    // held in registers (the opaque move keeps the compiler from forming them again for every step)
     uint32_t K2[8], K4[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -217,24 +264,13 @@ __device__ void draw_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, u
         const int item = __shfl_sync(0xffffffffu, take(), 0);
         if (item >= items) break;
         const int hs = item / per, first = (item - hs * per) * ITEM;
-        const uint32_t sweep = sweep0 + (uint32_t)(hs >> 1);
-        if (d.tiles > 1 && (hs & 1) == 0 && first == 0 && lane == 0) {
-            const int64_t N = (int64_t)d.L * d.L;
-            d.hist[2 * (int64_t)sweep] = -N;
-            d.hist[2 * (int64_t)sweep + 1] = -2 * N;
-        }
-        const PhiloxWordConsts pc = philox_consts(d.key, 0u, sweep, (uint32_t)(hs & 1));
-        if (first + ITEM <= d.words) {
-#pragma unroll 1
-            for (int k = 0; k < ITEM; k += 32 * G) draw_words<G, true>(w, pc, hs, first + k, K2, K4);
-        } else {
-#pragma unroll 1
-            for (int word0 = first; word0 < d.words; word0 += 32) draw_words<1, false>(w, pc, hs, word0, K2, K4);
-        }
+        if (d.tiles > 1 && (hs & 1) == 0 && first == 0 && lane == 0)
+            open_entry(d.hist, sweep0 + (uint32_t)(hs >> 1), d.L);
+        draw_step<G, ITEM>(w, one, 0, hs, first, K2, K4, lattice, bits);
     }
     while (w.qn > 0) {
         __syncwarp();
-        drain_draws(w, min(w.qn, 32));
+        drain_draws(w, min(w.qn, 32), lattice, bits);
     }
     __syncwarp();
 }
@@ -639,6 +675,184 @@ __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ A
                                   [&] { return lane == 0 ? atomicAdd(&d.ticket[st.gen_buf], 1) : 0; });
 }
 
+// ---- batches: the same for many lattices of a batch, in common launches.  The geometry of each
+// lattice's tiles follows from its side and the batch's chunk, and its places in the mask
+// buffers, the copies of the planes and the launch's tables from the plane words of the
+// lattices before it, so a change of the batch costs three small tables.
+
+// dense: the batch has work for every SM throughout a launch, so tiles are as tall as strips of
+// 16 rows make them (few halo rows) and lattices of up to 512 are one tile; else they are low,
+// for short half-sweeps.
+__host__ __device__ inline bool batch_whole(int W, int dense) { return W <= 3 || (dense && W <= 8); }
+
+__host__ __device__ inline void batch_geometry(int W, int chunk, int dense, AheadPlan& p)
+{
+    const int L = 64 * W, most = kStrips / W;  // strips one above the other
+    p.strip = 2;
+    if (batch_whole(W, dense)) {
+        while (L > most * p.strip) p.strip *= 2;
+        p.groups = L / p.strip;
+        p.rows = L;
+        p.halo = 0;
+        p.tiles = 1;
+        return;
+    }
+    // not dense: the shortest strips that leave a tile at least as many own rows as halo rows
+    while (p.strip < kMaxStrip && (dense || most * p.strip < 8 * chunk)) p.strip *= 2;
+    p.groups = most;
+    p.halo = 2 * chunk;
+    p.rows = p.groups * p.strip - 2 * p.halo;
+    p.tiles = (L + p.rows - 1) / p.rows;
+}
+
+// Entry of a table of prefix sums that holds `at`.
+__device__ __forceinline__ int find_entry(const int32_t* start, int count, int at)
+{
+    int lo = 0, hi = count;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (start[mid] <= at)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+// Sweeps of a run of `total` that lattice d takes part in: up to its own limit.
+__device__ __forceinline__ int sweeps_of(const LatticeDesc& d, int total)
+{
+    if (!d.active || d.sweep >= d.target) return 0;
+    const uint32_t left = d.target - d.sweep;
+    return left < (uint32_t)total ? (int)left : total;
+}
+
+__device__ __forceinline__ AheadLattice batch_lattice(const AheadBatch& b, const LatticeDesc& d, int word_start)
+{
+    AheadPlan p;
+    batch_geometry(d.W, b.chunk, b.dense, p);
+    AheadLattice a;
+    a.home = d.plane[0];
+    a.copy = b.copy + 4 * (size_t)word_start;
+    a.masks[0] = b.masks[0] + 2 * (size_t)b.chunk * word_start;
+    a.masks[1] = b.masks[1] + 2 * (size_t)b.chunk * word_start;
+    a.ticket = nullptr;
+    a.hist = d.hist;
+    a.status = b.status;
+    a.key = d.key;
+    a.t2 = d.t2;
+    a.t4 = d.t4;
+    a.all2 = d.all2;
+    a.all4 = d.all4;
+    a.L = d.L;
+    a.W = d.W;
+    a.words = d.L * d.W;
+    a.strip = p.strip;
+    a.groups = p.groups;
+    a.rows = p.rows;
+    a.halo = p.halo;
+    a.tiles = p.tiles;
+    return a;
+}
+
+__global__ void __launch_bounds__(kNT, 1) ahead_batch_kernel(const __grid_constant__ AheadBatch b, const AheadBatchStep st)
+{
+    extern __shared__ __align__(16) unsigned char smem_ahead[];
+    SharedAhead& sh = *reinterpret_cast<SharedAhead*>(smem_ahead);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_launch_next();
+    grid_wait();
+    // the tables behind the few sums that a chunk needs
+    int32_t* const tile_start = reinterpret_cast<int32_t*>(sh.sums) + 2 * kMaxBatchChunk;
+    int32_t* const step_start = tile_start + b.count + 1;
+    int32_t* const word_start = step_start + b.count + 1;
+    for (int k = threadIdx.x; k < 3 * (b.count + 1); k += kNT) tile_start[k] = b.tables[k];
+    __syncthreads();
+
+    if (st.upd_n > 0 || st.fill)
+        for (int tile = (int)blockIdx.x; tile < b.tiles; tile += (int)gridDim.x) {
+            const int l = find_entry(tile_start, b.count, tile);
+            const int local = tile - tile_start[l];
+            if (threadIdx.x == 0) {
+                const LatticeDesc& ld = b.desc[l];
+                const int mine = sweeps_of(ld, st.total);
+                AheadLattice& d = sh.now.lattice;
+                AheadStep& s = sh.now.step;
+                d = batch_lattice(b, ld, word_start[l]);
+                s.upd_n = st.fill ? mine : max(0, min(mine - st.upd_off, st.upd_n));
+                s.upd_sweep = ld.sweep + (uint32_t)st.upd_off;
+                s.upd_buf = st.upd_buf;
+                s.src = d.tiles > 1 ? st.src : -1;
+                s.dst = d.tiles > 1 && st.upd_off + s.upd_n < mine ? st.src ^ 1 : -1;
+                s.alone = 0;
+            }
+            __syncthreads();
+            const AheadLattice& d = sh.now.lattice;
+            const AheadStep& s = sh.now.step;
+            if (s.upd_n == 0) {
+            } else if (st.fill) {
+                // the first launch of a run: the copy of the planes that the first update reads
+                const int from = local * d.rows * d.W, n = d.tiles > 1 ? min(d.rows * d.W, d.words - from) : 0;
+                for (int k = threadIdx.x; k < n; k += kNT) {
+                    d.copy[from + k] = d.home[from + k];
+                    d.copy[d.words + from + k] = d.home[d.words + from + k];
+                }
+            } else if (d.strip == 2) {
+                update_tile<2>(d, s, local, sh);
+            } else if (d.strip == 4) {
+                update_tile<4>(d, s, local, sh);
+            } else if (d.strip == 8) {
+                update_tile<8>(d, s, local, sh);
+            } else {
+                update_tile<16>(d, s, local, sh);
+            }
+            __syncthreads();
+        }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        b.ticket[st.gen_buf ^ 1] = 0;
+        if (st.gen_n == 0) b.ticket[st.gen_buf] = 0;
+    }
+    if (st.gen_n == 0) return;
+
+    DrawState w{&sh.queue[warp], 0, lane};
+    uint2* const masks = b.masks[st.gen_buf];
+    auto lattice = [&](int l) {
+        const LatticeDesc& d = b.desc[l];
+        return DrawLattice{d.key, d.t2, d.t4, d.all2, d.all4, d.L * d.W, d.sweep + (uint32_t)st.gen_off,
+                           masks + 2 * (size_t)b.chunk * word_start[l]};
+    };
+    auto bits = [&](const DrawLattice& d, uint32_t c, uint4& b2, uint4& b4) {
+        const uint32_t t2 = d.t2 << (4u * c), t4 = d.t4 << (4u * c);
+        b2 = make_uint4(plane_mask(t2, 0), plane_mask(t2, 1), plane_mask(t2, 2), plane_mask(t2, 3));
+        b4 = make_uint4(plane_mask(t4, 0), plane_mask(t4, 1), plane_mask(t4, 2), plane_mask(t4, 3));
+    };
+    const int per = step_start[b.count], items = 2 * st.gen_n * per;
+    for (;;) {
+        int item = 0;
+        if (lane == 0) item = atomicAdd(&b.ticket[st.gen_buf], 1);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if (item >= items) break;
+        const int hs = item / per, r = item - hs * per;
+        const int l = find_entry(step_start, b.count, r);
+        const LatticeDesc& ld = b.desc[l];
+        if (st.gen_off + (hs >> 1) >= sweeps_of(ld, st.total)) continue;
+        const int first = (r - step_start[l]) * kItemWords;
+        const DrawLattice d = lattice(l);
+        if (!batch_whole(ld.W, b.dense) && (hs & 1) == 0 && first == 0 && lane == 0) open_entry(ld.hist, d.sweep0 + (uint32_t)(hs >> 1), ld.L);
+        uint32_t K2[8], K4[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            K2[k] = plane_mask(d.t2, k);
+            K4[k] = plane_mask(d.t4, k);
+        }
+        draw_step<4, kItemWords>(w, d, l, hs, first, K2, K4, lattice, bits);
+    }
+    while (w.qn > 0) {
+        __syncwarp();
+        drain_draws(w, min(w.qn, 32), lattice, bits);
+    }
+}
+
 template <int K>
 cudaError_t launch_k(const AheadLattice& d, const AheadStep& st, int grid, cudaStream_t s)
 {
@@ -663,6 +877,62 @@ cudaError_t launch_step(const AheadLattice& d, const AheadStep& st, cudaStream_t
 }
 
 }  // namespace
+
+// Sides up to 4,096 (longer rows leave a tile too few own rows) and as many lattices as the
+// tables in shared memory hold.
+int ahead_batch_max_L() { return 4096; }
+int ahead_batch_max_count() { return (2 * kMaxChunk - 2 * kMaxBatchChunk) / 3 - 1; }
+
+// Sweeps of a launch for a batch whose longest side is L: the tallest tile that W words a row
+// allow is four times as high as its halo.
+int ahead_batch_chunk(int64_t L)
+{
+    const int held = kStrips / (int)(L / 64) * kMaxStrip;
+    return std::max(1, std::min(16, held / 8));
+}
+
+int32_t ahead_batch_tiles(int64_t L, int chunk, int dense)
+{
+    AheadPlan p;
+    batch_geometry((int)(L / 64), chunk, dense, p);
+    return p.tiles;
+}
+
+int32_t ahead_batch_steps(int64_t L) { return (int32_t)((L * (L / 64) + kItemWords - 1) / kItemWords); }
+
+cudaError_t ahead_batch_configure()
+{
+    return cudaFuncSetAttribute(ahead_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SharedAhead));
+}
+
+cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s)
+{
+    // chunk k is drawn by the launch that updates chunk k - 1, as for a single lattice
+    int64_t drawn = 0, updated = 0;
+    int in_flight = 0, k = 0;
+    AheadBatchStep st;
+    st.total = (int32_t)n;
+    while (updated < n) {
+        const int next = (int)std::min<int64_t>(n - drawn, b.chunk);
+        st.upd_off = (int32_t)updated;
+        st.upd_n = in_flight;
+        st.upd_buf = (k & 1) ^ 1;
+        st.gen_off = (int32_t)drawn;
+        st.gen_n = next;
+        st.gen_buf = k & 1;
+        st.src = (k & 1) ^ 1;
+        st.fill = k == 0;
+        const int64_t want = std::max<int64_t>(b.tiles, 0) + (2 * next * steps + kWarps - 1) / kWarps;
+        const int grid = (int)std::min<int64_t>(sm_count(), want);
+        const cudaError_t e = launch_following(ahead_batch_kernel, dim3(grid), dim3(kNT), sizeof(SharedAhead), s, b, st);
+        if (e != cudaSuccess) return e;
+        updated += in_flight;
+        drawn += next;
+        in_flight = next;
+        ++k;
+    }
+    return cudaSuccess;
+}
 
 int ahead_max_L() { return 8192; }
 

@@ -81,3 +81,47 @@ def test_planes_set_between_runs():
     assert np.array_equal(m, M) and np.array_equal(e, E)
     assert np.array_equal(lat.get_lattice(), ref)
     lat.close()
+
+
+def batch_of(Ls, limits, mode=ising.CLUSTER_AUTO):
+    b = ising.Batch(len(Ls) + 2, max(Ls), sum(L * L // 8 + 16 * n + 4096 for L, n in zip(Ls, limits)) + (1 << 22))
+    b.set_cluster(mode)
+    betas = [0.3 + 0.05 * (k % 7) for k in range(len(Ls))]
+    idx = [b.add(L, be, 50 + k, ising.HOT if k % 2 else ising.COLD, n)
+           for k, (L, be, n) in enumerate(zip(Ls, betas, limits))]
+    return b, betas, idx
+
+
+def test_batch_matches_oracle():
+    # one-tile lattices (strips of 2 and 4 rows) and lattices of several tiles; limits inside a
+    # chunk, at its end and beyond the runs; runs shorter and longer than a chunk of 16 sweeps
+    Ls = [64, 128, 192, 256, 320, 384, 448, 512, 1088]
+    limits = [200, 16, 33, 200, 47, 48, 200, 20, 200]
+    b, betas, idx = batch_of(Ls, limits)
+    for n in (16, 5, 32, 1):
+        b.run(n)
+    for k, L in enumerate(Ls):
+        done = min(limits[k], 54)
+        ref, M, E, _ = oracle.run(L, betas[k], 50 + k, ising.HOT if k % 2 else ising.COLD, done)
+        m, e = b.history(idx[k])
+        assert b.sweeps_done(idx[k]) == done
+        assert np.array_equal(m, M) and np.array_equal(e, E), L
+        assert np.array_equal(b.get_lattice(idx[k]), ref), L
+    b.close()
+
+
+@pytest.mark.parametrize("Ls", [[4096, 64, 2112], [2048, 960, 1536, 1344], [3072, 1024, 128, 640]])
+def test_batch_matches_tiled(Ls):
+    out = []
+    for mode in (ising.CLUSTER_AUTO, ising.CLUSTER_OFF):
+        b, _, idx = batch_of(Ls, [60] * len(Ls), mode)
+        for n in (20, 7):
+            b.run(n)
+        # a lattice leaves and another joins between runs (its slot and places are reused)
+        b.remove(idx[1])
+        new = b.add(320, 0.41, 99, ising.HOT, 60)
+        b.run(17)
+        out.append([(b.history(i), b.get_lattice(i)) for i in (idx[0], idx[2], new)])
+        b.close()
+    for ((ma, ea), la), ((mt, et), lt) in zip(*out):
+        assert np.array_equal(ma, mt) and np.array_equal(ea, et) and np.array_equal(la, lt)
