@@ -16,6 +16,7 @@
 #include "arena.h"
 #include "ising_internal.cuh"
 #include "jit.h"
+#include "readback.h"
 #include "sweep3d.cuh"
 
 using namespace ising;
@@ -383,16 +384,21 @@ struct Engine {
         return ISING_OK;
     }
 
+    // What a report read as the status word: an error, and the word cleared, unless it is OK.
+    int judge(int64_t st)
+    {
+        if (st == kStatusOk) return ISING_OK;
+        CK(cudaMemsetAsync(d_status, 0, sizeof(int), stream));
+        return fail(ISING_ETIMEOUT, "sweep kernel reported status %d (bounded wait expired)", (int)st);
+    }
+
     int check_status()
     {
-        int st = 0;
-        CK(cudaMemcpyAsync(&st, d_status, sizeof(int), cudaMemcpyDeviceToHost, stream));
+        PinnedBlock blk;
+        if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+        CK(launch_report(nullptr, nullptr, 0, 0, d_status, blk.words(), stream));
         CK(cudaStreamSynchronize(stream));
-        if (st != kStatusOk) {
-            CK(cudaMemsetAsync(d_status, 0, sizeof(int), stream));
-            return fail(ISING_ETIMEOUT, "sweep kernel reported status %d (bounded wait expired)", st);
-        }
-        return ISING_OK;
+        return judge(blk.words()[0]);
     }
 
     void destroy()
@@ -444,8 +450,17 @@ struct Arena : FreeList {
 
 void ising::set_last_error(const char* msg) { t_error = msg; }
 
+namespace {
+// A handle's or batch's share in the page-locked blocks (readback.cu).
+struct ReadbackUser {
+    ReadbackUser() { readback_user(1); }
+    ~ReadbackUser() { readback_user(-1); }
+};
+}  // namespace
+
 // ====================================================================== handles
 struct ising_s {
+    ReadbackUser readback;
     int64_t L = 0;
     double beta = 0;
     uint64_t seed = 0;
@@ -463,8 +478,8 @@ struct ising_s {
     int64_t sweeps_done = 0;
     int64_t* d_me0 = nullptr;   // start-state (M, E)
     unsigned long long* d_work3 = nullptr;  // 3D: the half-sweeps' work counters (one per colour)
-    double* d_mom = nullptr;    // 6 doubles
-    uint64_t* d_sums = nullptr; // 11 limbs
+    int8_t* d_read = nullptr;   // int8 rows on their way to the host (ReadBuffer)
+    int64_t d_read_bytes = 0;
     std::string kernel_note;    // which sweep kernel runs, and why (ising_specialized)
     AheadLattice ahead{};       // packed, built-in kernel, L <= ahead_max_L(): the sweep with its
     AheadPlan ahead_plan;       // random numbers drawn ahead (tiles = 0: the tiled kernel)
@@ -474,6 +489,7 @@ struct ising_s {
 };
 
 struct ising_batch_s {
+    ReadbackUser readback;
     struct Slot {
         bool used = false;
         int64_t L = 0;
@@ -505,8 +521,8 @@ struct ising_batch_s {
     std::vector<Slot> slots;
     int32_t count = 0;
     int64_t* d_me = nullptr;
-    double* d_mom = nullptr;
-    uint64_t* d_sums = nullptr;
+    int8_t* d_read = nullptr;
+    int64_t d_read_bytes = 0;
 };
 
 namespace {
@@ -630,26 +646,55 @@ CubicDesc cubic_desc(ising_t h)
     return d;
 }
 
+// Device buffer for int8 rows on their way to the host: up to 32 MB of it stay with the handle or
+// batch (allocating and freeing it for each call costs 0.1 ms, which is what the rows of a
+// lattice of L = 1,024 take), more is held for the call only.
+struct ReadBuffer {
+    static constexpr int64_t kKept = 32ll << 20;
+    int8_t* p = nullptr;
+    bool own = false;
+    cudaError_t open(int8_t** keep, int64_t* keep_bytes, int64_t bytes)
+    {
+        if (bytes <= *keep_bytes) {
+            p = *keep;
+            return cudaSuccess;
+        }
+        if (bytes > kKept) {
+            own = true;
+            return cudaMalloc(&p, (size_t)bytes);
+        }
+        cudaFree(*keep);
+        *keep = nullptr;
+        *keep_bytes = 0;
+        const cudaError_t e = cudaMalloc(&p, (size_t)bytes);
+        if (e == cudaSuccess) {
+            *keep = p;
+            *keep_bytes = bytes;
+        }
+        return e;
+    }
+    ~ReadBuffer()
+    {
+        if (own) cudaFree(p);
+    }
+};
+
 // int8 copy of a cubic lattice, index (i*L + j)*L + k, through a bounded staging buffer.
 // Rows [row0, row0 + nrows) (row r = i*L + j, L sites each) of a cube into out.
 int cubic_rows_to_host(ising_t h, int64_t row0, int64_t nrows, int8_t* out)
 {
     const int64_t L = h->L;
     const int64_t chunk = std::min<int64_t>(nrows, std::max<int64_t>(1, (int64_t)(256ll << 20) / L));
-    int8_t* tmp = nullptr;
-    CK(cudaMalloc(&tmp, (size_t)(chunk * L)));
+    ReadBuffer tmp;
+    CK(tmp.open(&h->d_read, &h->d_read_bytes, chunk * L));
     for (int64_t r0 = 0; r0 < nrows; r0 += chunk) {
         const int64_t nr = std::min<int64_t>(chunk, nrows - r0);
         cudaError_t e =
-            launch_cubic_unpack(h->planes, h->planes + plane_words(h), tmp, L, row0 + r0, nr, h->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out + r0 * L, tmp, (size_t)(nr * L), cudaMemcpyDeviceToHost, h->stream);
+            launch_cubic_unpack(h->planes, h->planes + plane_words(h), tmp.p, L, row0 + r0, nr, h->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(out + r0 * L, tmp.p, (size_t)(nr * L), cudaMemcpyDeviceToHost, h->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-        if (e != cudaSuccess) {
-            cudaFree(tmp);
-            return cuda_fail(e, "cubic unpack to host");
-        }
+        if (e != cudaSuccess) return cuda_fail(e, "cubic unpack to host");
     }
-    cudaFree(tmp);
     return ISING_OK;
 }
 
@@ -662,32 +707,39 @@ int read_status(ising_t h)
     return ISING_OK;
 }
 
+// The handle's status word on the device (its sweeps may give up a bounded wait), or null.
+const int* status_word(ising_t h) { return h->kernel == ISING_PACKED ? h->eng.d_status : nullptr; }
+
+// Waits for the stream and judges the status a report put into st.
+int await_report(ising_t h, const int64_t* st)
+{
+    CK(cudaStreamSynchronize(h->stream));
+    return h->kernel == ISING_PACKED ? h->eng.judge(*st) : ISING_OK;
+}
+
 // Copies the lattice to host int8 through a bounded device staging buffer.
 // Rows [row0, row0 + nrows) of a packed lattice as int8 spins into out (nrows * L bytes).
 int packed_rows_to_host(const uint32_t* black, const uint32_t* white, int64_t L, int64_t row0, int64_t nrows,
-                        int8_t* out, cudaStream_t s)
+                        int8_t* out, cudaStream_t s, int8_t** keep, int64_t* keep_bytes)
 {
     const int64_t rows_per = std::max<int64_t>(1, (int64_t)(256ll << 20) / L);
     const int64_t chunk_rows = std::min<int64_t>(nrows, rows_per);
-    int8_t* tmp = nullptr;
-    CK(cudaMalloc(&tmp, (size_t)(chunk_rows * L)));
+    ReadBuffer tmp;
+    CK(tmp.open(keep, keep_bytes, chunk_rows * L));
     for (int64_t r0 = 0; r0 < nrows; r0 += chunk_rows) {
         const int64_t nr = std::min<int64_t>(chunk_rows, nrows - r0);
-        cudaError_t e = launch_unpack(black, white, tmp, L, row0 + r0, nr, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out + r0 * L, tmp, (size_t)(nr * L), cudaMemcpyDeviceToHost, s);
+        cudaError_t e = launch_unpack(black, white, tmp.p, L, row0 + r0, nr, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(out + r0 * L, tmp.p, (size_t)(nr * L), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) {
-            cudaFree(tmp);
-            return cuda_fail(e, "unpack to host");
-        }
+        if (e != cudaSuccess) return cuda_fail(e, "unpack to host");
     }
-    cudaFree(tmp);
     return ISING_OK;
 }
 
-int packed_to_host(const uint32_t* black, const uint32_t* white, int64_t L, int8_t* out, cudaStream_t s)
+int packed_to_host(const uint32_t* black, const uint32_t* white, int64_t L, int8_t* out, cudaStream_t s, int8_t** keep,
+                   int64_t* keep_bytes)
 {
-    return packed_rows_to_host(black, white, L, 0, L, out, s);
+    return packed_rows_to_host(black, white, L, 0, L, out, s, keep, keep_bytes);
 }
 
 int host_to_packed(const int8_t* in, uint32_t* black, uint32_t* white, int64_t L, cudaStream_t s)
@@ -741,8 +793,7 @@ void destroy_handle(ising_t h)
     cudaFree(h->d_me0);
     cudaFree(h->d_work3);
     cudaFree(h->ahead_ws);
-    cudaFree(h->d_mom);
-    cudaFree(h->d_sums);
+    cudaFree(h->d_read);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
 }
@@ -804,8 +855,6 @@ int ising_init_ex(ising_t* out, int64_t L, double beta, uint64_t seed, int start
         }                                         \
     } while (0)
     CKH(cudaMalloc(&h->d_me0, 2 * sizeof(int64_t)));
-    CKH(cudaMalloc(&h->d_mom, 6 * sizeof(double)));
-    CKH(cudaMalloc(&h->d_sums, 11 * sizeof(uint64_t)));
     if (kernel == ISING_PACKED) {
         const int64_t plane_words = L * (L / 64);
         CKH(cudaMalloc(&h->planes, sizeof(uint32_t) * 2 * (size_t)plane_words));
@@ -957,8 +1006,6 @@ int ising_init3d(ising_t* out, int64_t L, double beta, uint64_t seed, int start,
             h->kernel_note = "built-in: " + why;
     }
     cudaError_t e = cudaMalloc(&h->d_me0, 2 * sizeof(int64_t));
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_mom, 6 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_sums, 11 * sizeof(uint64_t));
     if (e == cudaSuccess) e = cudaMalloc(&h->planes, sizeof(uint32_t) * 2 * (size_t)plane_words(h));
     if (e == cudaSuccess) e = cudaMalloc(&h->d_work3, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_work3, 0, 2 * sizeof(unsigned long long), h->stream);
@@ -1033,11 +1080,13 @@ int ising_observables(ising_t h, int64_t* M, int64_t* E, int64_t* sweeps_done)
 {
     int rc = check_handle(h);
     if (rc) return rc;
-    int64_t me[2];
+    PinnedBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
     const int64_t* src = h->sweeps_done ? h->hist + 2 * (h->sweeps_done - 1) : h->d_me0;
-    CK(cudaMemcpyAsync(me, src, sizeof(me), cudaMemcpyDeviceToHost, h->stream));
-    rc = read_status(h);
+    CK(launch_report(nullptr, src, 0, 1, status_word(h), blk.words(), h->stream));
+    rc = await_report(h, blk.words());
     if (rc) return rc;
+    const int64_t* me = blk.words() + 2;
     if (M) *M = me[0];
     if (E) *E = me[1];
     if (sweeps_done) *sweeps_done = h->sweeps_done;
@@ -1051,14 +1100,25 @@ int ising_history(ising_t h, int64_t first, int64_t count, int64_t* M, int64_t* 
     if (first < 0 || count < 0 || first > h->sweeps_done || count > h->sweeps_done - first)
         return fail(ISING_EINVAL, "history range [%lld, %lld) beyond %lld sweeps", (long long)first,
                     (long long)(first + count), (long long)h->sweeps_done);
-    std::vector<int64_t> buf(2 * (size_t)count);
-    if (count) CK(cudaMemcpyAsync(buf.data(), h->hist + 2 * first, sizeof(int64_t) * buf.size(),
-                                  cudaMemcpyDeviceToHost, h->stream));
-    rc = read_status(h);
+    std::vector<int64_t> buf;
+    const int64_t* e;
+    PinnedBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+    if (count <= PinnedBlock::kEntries) {
+        CK(launch_report(nullptr, h->hist, first, count, status_word(h), blk.words(), h->stream));
+        rc = await_report(h, blk.words());
+        e = blk.words() + 2;
+    } else {
+        buf.resize(2 * (size_t)count);
+        CK(cudaMemcpyAsync(buf.data(), h->hist + 2 * first, sizeof(int64_t) * buf.size(), cudaMemcpyDeviceToHost,
+                           h->stream));
+        rc = read_status(h);
+        e = buf.data();
+    }
     if (rc) return rc;
     for (int64_t k = 0; k < count; ++k) {
-        if (M) M[k] = buf[2 * k];
-        if (E) E[k] = buf[2 * k + 1];
+        if (M) M[k] = e[2 * k];
+        if (E) E[k] = e[2 * k + 1];
     }
     return ISING_OK;
 }
@@ -1069,15 +1129,16 @@ int ising_moments_ex(ising_t h, int64_t burn_in, double out[6], uint64_t sums[11
     if (rc) return rc;
     if (!out) return fail(ISING_EINVAL, "null output");
     if (burn_in < 0 || burn_in >= h->sweeps_done) return fail(ISING_EINVAL, "no samples after burn-in");
-    CK(launch_moments(h->hist, burn_in, h->sweeps_done - burn_in, site_count(h), h->d_mom, h->d_sums, h->stream));
-    double m[6];
-    uint64_t s[11];
-    CK(cudaMemcpyAsync(m, h->d_mom, sizeof(m), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(s, h->d_sums, sizeof(s), cudaMemcpyDeviceToHost, h->stream));
-    rc = read_status(h);
+    PinnedBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+    double* m = reinterpret_cast<double*>(blk.words() + 2);
+    uint64_t* t = reinterpret_cast<uint64_t*>(blk.words() + 8);
+    CK(launch_moments(nullptr, h->hist, burn_in, h->sweeps_done - burn_in, site_count(h), m, t, status_word(h),
+                      blk.words(), h->stream));
+    rc = await_report(h, blk.words());
     if (rc) return rc;
-    memcpy(out, m, sizeof(m));
-    if (sums) memcpy(sums, s, sizeof(s));
+    memcpy(out, m, 6 * sizeof(double));
+    if (sums) memcpy(sums, t, 11 * sizeof(uint64_t));
     return ISING_OK;
 }
 
@@ -1103,7 +1164,8 @@ int ising_get_lattice(ising_t h, int8_t* out)
     if (rc) return rc;
     if (h->kernel == kKernelCubic) return cubic_to_host(h, out);
     if (h->kernel == ISING_PACKED)
-        return packed_to_host(h->planes, h->planes + h->L * (h->L / 64), h->L, out, h->stream);
+        return packed_to_host(h->planes, h->planes + h->L * (h->L / 64), h->L, out, h->stream, &h->d_read,
+                              &h->d_read_bytes);
     CK(cudaMemcpyAsync(out, h->lat, (size_t)(h->L * h->L), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return ISING_OK;
@@ -1123,7 +1185,8 @@ int ising_get_rows(ising_t h, int64_t row0, int64_t nrows, int8_t* out)
     if (rc) return rc;
     if (h->kernel == kKernelCubic) return cubic_rows_to_host(h, row0, nrows, out);
     if (h->kernel == ISING_PACKED)
-        return packed_rows_to_host(h->planes, h->planes + L * (L / 64), L, row0, nrows, out, h->stream);
+        return packed_rows_to_host(h->planes, h->planes + L * (L / 64), L, row0, nrows, out, h->stream, &h->d_read,
+                                   &h->d_read_bytes);
     CK(cudaMemcpyAsync(out, h->lat + row0 * L, (size_t)(nrows * L), cudaMemcpyDeviceToHost, h->stream));
     CK(cudaStreamSynchronize(h->stream));
     return ISING_OK;
@@ -1158,6 +1221,18 @@ int ising_get_planes(ising_t h, uint32_t* black, uint32_t* white)
     if (rc) return rc;
     if (h->kernel == ISING_INT8) return fail(ISING_EINVAL, "not a packed handle");
     const size_t bytes = sizeof(uint32_t) * (size_t)plane_words(h);
+    if (2 * bytes + 16 <= (size_t)PinnedBlock::kBytes) {
+        PinnedBlock blk;
+        if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+        uint32_t* w = static_cast<uint32_t*>(blk.p);
+        w[0] = w[1] = 0u;
+        CK(launch_report_words(h->planes, 2 * plane_words(h), status_word(h), w, h->stream));
+        rc = await_report(h, blk.words());
+        if (rc) return rc;
+        if (black) memcpy(black, w + 4, bytes);
+        if (white) memcpy(white, w + 4 + plane_words(h), bytes);
+        return ISING_OK;
+    }
     if (black) CK(cudaMemcpyAsync(black, h->planes, bytes, cudaMemcpyDeviceToHost, h->stream));
     if (white) CK(cudaMemcpyAsync(white, h->planes + plane_words(h), bytes, cudaMemcpyDeviceToHost, h->stream));
     return read_status(h);
@@ -1517,13 +1592,22 @@ int check_batch(ising_batch_t b, int32_t idx)
     return ISING_OK;
 }
 
+// One report of slot idx: its sweep count, and count history entries from `first` on (left out
+// where they lie beyond that).
+int batch_report(ising_batch_t b, int32_t idx, int64_t first, int64_t count, const PinnedBlock& blk)
+{
+    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+    CK(launch_report(b->eng.d_desc + idx, nullptr, first, count, b->eng.d_status, blk.words(), b->stream));
+    CK(cudaStreamSynchronize(b->stream));
+    return b->eng.judge(blk.words()[0]);
+}
+
 int batch_sweeps_done(ising_batch_t b, int32_t idx, int64_t* done)
 {
-    uint32_t sw = 0;
-    CK(cudaMemcpyAsync(&sw, &b->eng.d_desc[idx].sweep, sizeof(uint32_t), cudaMemcpyDeviceToHost, b->stream));
-    int rc = b->eng.check_status();
+    PinnedBlock blk;
+    int rc = batch_report(b, idx, 0, 0, blk);
     if (rc) return rc;
-    *done = sw;
+    *done = blk.words()[1];
     return ISING_OK;
 }
 }  // namespace
@@ -1560,8 +1644,6 @@ int ising_batch_create_ex(ising_batch_t* out, int32_t capacity, int64_t max_L, i
     if (!rc) rc = b->arena.init(arena_bytes);
     if (!rc) {
         cudaError_t e = cudaMalloc(&b->d_me, 2 * sizeof(int64_t));
-        if (e == cudaSuccess) e = cudaMalloc(&b->d_mom, 6 * sizeof(double));
-        if (e == cudaSuccess) e = cudaMalloc(&b->d_sums, 11 * sizeof(uint64_t));
         if (e != cudaSuccess) rc = cuda_fail(e, "batch buffers");
     }
     if (!rc) rc = rebuild_tiles(b);
@@ -1829,18 +1911,17 @@ int ising_batch_observables_ex(ising_batch_t b, int32_t idx, int64_t* M, int64_t
 {
     int rc = check_batch(b, idx);
     if (rc) return rc;
-    int64_t done = 0;
-    rc = batch_sweeps_done(b, idx, &done);
+    PinnedBlock blk;
+    rc = batch_report(b, idx, kLastEntry, 1, blk);
     if (rc) return rc;
-    const auto& d = b->slots[idx].desc;
-    int64_t me[2];
+    const int64_t done = blk.words()[1];
     if (done == 0) {
+        const auto& d = b->slots[idx].desc;
         CK(launch_packed_observe(d.plane[0], d.plane[1], d.L, b->d_me, b->stream));
-        CK(cudaMemcpyAsync(me, b->d_me, sizeof(me), cudaMemcpyDeviceToHost, b->stream));
-    } else {
-        CK(cudaMemcpyAsync(me, d.hist + 2 * (done - 1), sizeof(me), cudaMemcpyDeviceToHost, b->stream));
+        CK(launch_report(nullptr, b->d_me, 0, 1, nullptr, blk.words(), b->stream));
+        CK(cudaStreamSynchronize(b->stream));
     }
-    CK(cudaStreamSynchronize(b->stream));
+    const int64_t* me = blk.words() + 2;
     if (M) *M = me[0];
     if (E) *E = me[1];
     if (sweeps_done) *sweeps_done = done;
@@ -1856,19 +1937,26 @@ int ising_batch_history(ising_batch_t b, int32_t idx, int64_t first, int64_t cou
 {
     int rc = check_batch(b, idx);
     if (rc) return rc;
-    int64_t done = 0;
-    rc = batch_sweeps_done(b, idx, &done);
+    // (a negative range asks the device for no entry and is refused below)
+    const bool small = first >= 0 && count >= 0 && count <= PinnedBlock::kEntries;
+    PinnedBlock blk;
+    rc = batch_report(b, idx, small ? first : 0, small ? count : 0, blk);
     if (rc) return rc;
+    const int64_t done = blk.words()[1];
     if (first < 0 || count < 0 || first > done || count > done - first)
         return fail(ISING_EINVAL, "history range beyond sweeps done");
-    std::vector<int64_t> buf(2 * (size_t)count);
-    const auto& d = b->slots[idx].desc;
-    if (count) CK(cudaMemcpyAsync(buf.data(), d.hist + 2 * first, sizeof(int64_t) * buf.size(),
-                                  cudaMemcpyDeviceToHost, b->stream));
-    CK(cudaStreamSynchronize(b->stream));
+    const int64_t* e = blk.words() + 2;
+    std::vector<int64_t> buf;
+    if (!small) {
+        buf.resize(2 * (size_t)count);
+        CK(cudaMemcpyAsync(buf.data(), b->slots[idx].desc.hist + 2 * first, sizeof(int64_t) * buf.size(),
+                           cudaMemcpyDeviceToHost, b->stream));
+        CK(cudaStreamSynchronize(b->stream));
+        e = buf.data();
+    }
     for (int64_t k = 0; k < count; ++k) {
-        if (M) M[k] = buf[2 * k];
-        if (E) E[k] = buf[2 * k + 1];
+        if (M) M[k] = e[2 * k];
+        if (E) E[k] = e[2 * k + 1];
     }
     return ISING_OK;
 }
@@ -1878,19 +1966,20 @@ int ising_batch_moments(ising_batch_t b, int32_t idx, int64_t burn_in, double ou
     int rc = check_batch(b, idx);
     if (rc) return rc;
     if (!out) return fail(ISING_EINVAL, "null output");
-    int64_t done = 0;
-    rc = batch_sweeps_done(b, idx, &done);
-    if (rc) return rc;
-    if (burn_in < 0 || burn_in >= done) return fail(ISING_EINVAL, "no samples after burn-in");
     const auto& d = b->slots[idx].desc;
-    CK(launch_moments(d.hist, burn_in, done - burn_in, (int64_t)d.L * d.L, b->d_mom, b->d_sums, b->stream));
-    double m[6];
-    uint64_t s[11];
-    CK(cudaMemcpyAsync(m, b->d_mom, sizeof(m), cudaMemcpyDeviceToHost, b->stream));
-    CK(cudaMemcpyAsync(s, b->d_sums, sizeof(s), cudaMemcpyDeviceToHost, b->stream));
+    PinnedBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+    double* m = reinterpret_cast<double*>(blk.words() + 2);
+    uint64_t* t = reinterpret_cast<uint64_t*>(blk.words() + 8);
+    // (a negative burn_in asks for no sample and is refused below)
+    CK(launch_moments(b->eng.d_desc + idx, nullptr, burn_in < 0 ? INT64_MAX : burn_in, 0, (int64_t)d.L * d.L, m, t,
+                      b->eng.d_status, blk.words(), b->stream));
     CK(cudaStreamSynchronize(b->stream));
-    memcpy(out, m, sizeof(m));
-    if (sums) memcpy(sums, s, sizeof(s));
+    rc = b->eng.judge(blk.words()[0]);
+    if (rc) return rc;
+    if (burn_in < 0 || burn_in >= blk.words()[1]) return fail(ISING_EINVAL, "no samples after burn-in");
+    memcpy(out, m, 6 * sizeof(double));
+    if (sums) memcpy(sums, t, 11 * sizeof(uint64_t));
     return ISING_OK;
 }
 
@@ -1902,7 +1991,7 @@ int ising_batch_get_lattice(ising_batch_t b, int32_t idx, int8_t* out)
     rc = b->eng.check_status();
     if (rc) return rc;
     const auto& d = b->slots[idx].desc;
-    return packed_to_host(d.plane[0], d.plane[1], d.L, out, b->stream);
+    return packed_to_host(d.plane[0], d.plane[1], d.L, out, b->stream, &b->d_read, &b->d_read_bytes);
 }
 
 int ising_batch_usage(ising_batch_t b, int64_t* arena_used, int32_t* slots_used)
@@ -1933,8 +2022,7 @@ int ising_batch_free(ising_batch_t b)
     cudaFree(b->ahead_ws);
     for (void* p : b->ahead_outgrown) cudaFree(p);
     cudaFree(b->d_me);
-    cudaFree(b->d_mom);
-    cudaFree(b->d_sums);
+    cudaFree(b->d_read);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
     return ISING_OK;

@@ -172,10 +172,12 @@ cudaError_t launch_int8_half_sweep(int8_t* lat, int64_t L, uint64_t key, uint32_
                                    cudaStream_t s);
 cudaError_t launch_int8_observe(const int8_t* lat, int64_t L, int64_t* ME, cudaStream_t s);
 
-// Exact moments over hist[first .. first+count): writes 6 doubles
-// (abs_m, m2, m4, e, e2, binder) and the exact sums (see moments.cu).
-cudaError_t launch_moments(const int64_t* hist, int64_t first, int64_t count, int64_t N, double* out6,
-                           uint64_t* sums, cudaStream_t s);
+// Exact moments over hist[first .. first+count), or of the batch lattice desc over its samples from
+// `first` on: writes 6 doubles (abs_m, m2, m4, e, e2, binder) and the exact sums (see
+// moments.cu), nothing where there is no sample; report[0] = *status (0 for null), report[1] = the
+// sweep count.
+cudaError_t launch_moments(const LatticeDesc* desc, const int64_t* hist, int64_t first, int64_t count, int64_t N,
+                           double* out6, uint64_t* sums, const int* status, int64_t* report, cudaStream_t s);
 
 cudaError_t launch_philox_words(uint64_t key, const uint32_t* ctr4, int64_t n, uint32_t* out, cudaStream_t s);
 

@@ -36,9 +36,21 @@ __device__ double u128_to_double(const uint64_t* v)
     return (double)v[1] * 18446744073709551616.0 + (double)v[0];
 }
 
-__global__ void __launch_bounds__(kThreads) moments_kernel(const int64_t* hist, int64_t first, int64_t count,
-                                                           int64_t N, double* out6, uint64_t* sums_out)
+// desc: a batch lattice, whose history and sweep count are read from there (the samples then are
+// those from `first` on); report (may be null) receives the status word and the sweep count.
+__global__ void __launch_bounds__(kThreads) moments_kernel(const LatticeDesc* desc, const int64_t* hist, int64_t first,
+                                                           int64_t count, int64_t N, double* out6, uint64_t* sums_out,
+                                                           const int* status, int64_t* report)
 {
+    if (desc) {
+        hist = desc->hist;
+        count = (int64_t)desc->sweep - first;
+    }
+    if (report && threadIdx.x == 0) {
+        report[0] = status ? *status : 0;
+        report[1] = first + count;
+    }
+    if (count <= 0) return;  // refused by the caller
     __shared__ uint64_t sh[kLimbs][kThreads];
     uint64_t acc[kLimbs];
 #pragma unroll
@@ -123,10 +135,10 @@ __global__ void __launch_bounds__(kThreads) moments_kernel(const int64_t* hist, 
 
 }  // namespace
 
-cudaError_t launch_moments(const int64_t* hist, int64_t first, int64_t count, int64_t N, double* out6,
-                           uint64_t* sums, cudaStream_t s)
+cudaError_t launch_moments(const LatticeDesc* desc, const int64_t* hist, int64_t first, int64_t count, int64_t N,
+                           double* out6, uint64_t* sums, const int* status, int64_t* report, cudaStream_t s)
 {
-    moments_kernel<<<1, kThreads, 0, s>>>(hist, first, count, N, out6, sums);
+    moments_kernel<<<1, kThreads, 0, s>>>(desc, hist, first, count, N, out6, sums, status, report);
     return cudaGetLastError();
 }
 
