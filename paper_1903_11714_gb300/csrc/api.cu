@@ -550,10 +550,14 @@ int ensure_hist(ising_t h, int64_t need)
     return ISING_OK;
 }
 
+uint32_t thr32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : (uint32_t)T; }
+uint32_t all32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : 0u; }
+
 // The sweep with its random numbers drawn ahead: the lattice's plan and constants.
 int setup_ahead(ising_t h)
 {
-    const AheadPlan p = ahead_plan(h->L);
+    const bool cube = h->kernel == kKernelCubic;
+    const AheadPlan p = cube ? ahead_plan3(h->L) : ahead_plan(h->L);
     if (p.tiles == 0) return ISING_OK;
     CK(ahead_configure(p));
     h->ahead_plan = p;
@@ -561,13 +565,17 @@ int setup_ahead(ising_t h)
     a.home = h->planes;
     a.status = h->eng.d_status;
     a.key = h->seed;
-    a.t2 = h->desc.t2;
-    a.t4 = h->desc.t4;
-    a.all2 = h->desc.all2;
-    a.all4 = h->desc.all4;
+    a.t2 = thr32(h->T[0]);
+    a.t4 = thr32(h->T[1]);
+    a.t6 = thr32(h->T[2]);
+    a.all2 = all32(h->T[0]);
+    a.all4 = all32(h->T[1]);
+    a.all6 = all32(h->T[2]);
+    a.cube = p.cube;
     a.L = (int32_t)h->L;
-    a.W = (int32_t)(h->L / 64);
-    a.words = (int32_t)(h->L * (h->L / 64));
+    a.row_words = (int32_t)(h->L / 64);
+    a.W = cube ? a.L * a.row_words : a.row_words;
+    a.words = a.L * a.W;
     a.strip = p.strip;
     a.groups = p.groups;
     a.rows = p.rows;
@@ -624,9 +632,6 @@ int64_t plane_words(ising_t h)
 
 // Sites of the lattice: L^2 or L^3.
 int64_t site_count(ising_t h) { return (h->kernel == kKernelCubic ? h->L : 1) * h->L * h->L; }
-
-uint32_t thr32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : (uint32_t)T; }
-uint32_t all32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : 0u; }
 
 CubicDesc cubic_desc(ising_t h)
 {
@@ -702,19 +707,19 @@ int cubic_to_host(ising_t h, int8_t* out) { return cubic_rows_to_host(h, 0, h->L
 
 int read_status(ising_t h)
 {
-    if (h->kernel == ISING_PACKED) return h->eng.check_status();
+    if (h->kernel != ISING_INT8) return h->eng.check_status();
     CK(cudaStreamSynchronize(h->stream));
     return ISING_OK;
 }
 
 // The handle's status word on the device (its sweeps may give up a bounded wait), or null.
-const int* status_word(ising_t h) { return h->kernel == ISING_PACKED ? h->eng.d_status : nullptr; }
+const int* status_word(ising_t h) { return h->kernel != ISING_INT8 ? h->eng.d_status : nullptr; }
 
 // Waits for the stream and judges the status a report put into st.
 int await_report(ising_t h, const int64_t* st)
 {
     CK(cudaStreamSynchronize(h->stream));
-    return h->kernel == ISING_PACKED ? h->eng.judge(*st) : ISING_OK;
+    return h->kernel != ISING_INT8 ? h->eng.judge(*st) : ISING_OK;
 }
 
 // Copies the lattice to host int8 through a bounded device staging buffer.
@@ -1009,8 +1014,12 @@ int ising_init3d(ising_t* out, int64_t L, double beta, uint64_t seed, int start,
     if (e == cudaSuccess) e = cudaMalloc(&h->planes, sizeof(uint32_t) * 2 * (size_t)plane_words(h));
     if (e == cudaSuccess) e = cudaMalloc(&h->d_work3, 2 * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_work3, 0, 2 * sizeof(unsigned long long), h->stream);
+    if (e == cudaSuccess) e = cudaMalloc(&h->eng.d_status, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->eng.d_status, 0, sizeof(int), h->stream);
+    h->eng.stream = h->stream;
     if (e == cudaSuccess) e = launch_cubic_init(h->planes, h->planes + plane_words(h), L, seed, start, h->stream);
     rc = (e == cudaSuccess) ? ensure_hist(h, 1024) : cuda_fail(e, "3D lattice set-up");
+    if (!rc && !h->cubic_fixed[0]) rc = setup_ahead(h);
     if (!rc) rc = refresh_me0(h);
     if (!rc) {
         e = cudaStreamSynchronize(h->stream);

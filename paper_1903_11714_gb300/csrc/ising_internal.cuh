@@ -65,6 +65,7 @@ struct AheadPlan {
     int rows = 0, halo = 0;    // a tile's own rows, and extra rows above and below them
     int tiles = 0;
     int chunk = 0;             // most sweeps of one launch
+    int cube = 0;              // a cube: slices in the place of rows
     int64_t mask_bytes = 0;    // one buffer of acceptance masks (two are needed)
     int64_t copy_bytes = 0;    // both copies of the planes (0: the lattice is one tile)
 };
@@ -77,7 +78,9 @@ struct AheadLattice {
     int* status;               // set when a bounded wait runs out
     uint64_t key;
     uint32_t t2, t4, all2, all4;  // thresholds as in LatticeDesc
-    int32_t L, W, words;       // words: of one plane
+    int32_t L, W, words;       // words: of one plane (W: of a row, of a cube's slice)
+    uint32_t t6, all6;         // cubes
+    int32_t cube, row_words;   // cubes: 1, words of a row
     int32_t strip, groups, rows, halo, tiles;  // the plan's
 };
 // What one launch does: update upd_n sweeps from upd_sweep on from masks buffer upd_buf, reading
@@ -117,6 +120,7 @@ cudaError_t ahead_batch_configure();
 cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s);
 int ahead_max_L();
 AheadPlan ahead_plan(int64_t L);
+AheadPlan ahead_plan3(int64_t L);  // of a cube
 cudaError_t ahead_configure(const AheadPlan& p);
 // Whether n sweeps are one launch of one CTA that draws its own masks (no workspace needed).
 bool ahead_alone(const AheadLattice& d, int64_t n);

@@ -111,7 +111,26 @@ cudaError_t launch_cubic_observe(const uint32_t* black, const uint32_t* white, i
     return cudaGetLastError();
 }
 
-int cubic_words_per_group(int64_t L) { return (L / 64) % 4 == 0 ? 4 : 1; }
+// Adjacent words of a thread's group: its Philox calls overlap.  Three (rows of a multiple of three
+// words) only while a group's call indices share their high word, which a group of a power of
+// two does for any side.  us a sweep against one word a thread: L = 384 35.9 (2 words) / 47.2; 896
+// 255 (2) / 327; 576 90.8 (3) / 115; 960 292 (3) / 426 (and turns of 8).
+int cubic_words_per_group(int64_t L)
+{
+    const int64_t W = L / 64;
+    return W % 4 == 0 ? 4 : (W % 2 == 0 ? 2 : (W % 3 == 0 && cubic_q_small(L) ? 3 : 1));
+}
+
+template <int G>
+static cudaError_t launch_cubic_g(const CubicDesc& d, unsigned long long* work, int colour, uint32_t sweep, int grid,
+                                  cudaStream_t s)
+{
+    if (colour == 1)
+        return launch_following(cubic_half_sweep_kernel<kThreads3, G, true>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
+                                sweep, work);
+    return launch_following(cubic_half_sweep_kernel<kThreads3, G, false>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
+                            sweep, work);
+}
 
 cudaError_t launch_cubic_half_sweep(const CubicDesc& d, unsigned long long* work, int colour, uint32_t sweep,
                                     cudaStream_t s, const void* const* fixed)
@@ -128,17 +147,16 @@ cudaError_t launch_cubic_half_sweep(const CubicDesc& d, unsigned long long* work
         void* args[] = {&dd, &colour, &sweep, &work};
         return launch_following_c(fixed[colour], dim3(grid), dim3(kThreads3), 0, s, args);
     }
-    if (G == 4 && colour == 1)
-        return launch_following(cubic_half_sweep_kernel<kThreads3, 4, true>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
-                                sweep, work);
-    if (G == 4)
-        return launch_following(cubic_half_sweep_kernel<kThreads3, 4, false>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
-                                sweep, work);
-    if (colour == 1)
-        return launch_following(cubic_half_sweep_kernel<kThreads3, 1, true>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
-                                sweep, work);
-    return launch_following(cubic_half_sweep_kernel<kThreads3, 1, false>, dim3(grid), dim3(kThreads3), 0, s, d, colour,
-                            sweep, work);
+    switch (G) {
+    case 4:
+        return launch_cubic_g<4>(d, work, colour, sweep, grid, s);
+    case 3:
+        return launch_cubic_g<3>(d, work, colour, sweep, grid, s);
+    case 2:
+        return launch_cubic_g<2>(d, work, colour, sweep, grid, s);
+    default:
+        return launch_cubic_g<1>(d, work, colour, sweep, grid, s);
+    }
 }
 
 cudaError_t launch_cubic_unpack(const uint32_t* black, const uint32_t* white, int8_t* lat, int64_t L, int64_t row0,

@@ -221,8 +221,11 @@ __device__ __forceinline__ void block_add_twice(unsigned long long a, unsigned l
 // adds the fused observables; as a template parameter it leaves the colour-0 pass
 // without their instructions.
 //
-// Work order: each warp takes the next 8 x 32 word groups (rows in plane order) from
-// the counter work[colour] and its lanes walk them 32 consecutive groups at a time.
+// Work order: each warp takes the next 8 x 32 word groups (rows in plane order; fewer of a
+// cube too small to give every warp two turns of 8) and its lanes walk them 32 consecutive
+// groups at a time: its first turn by its own number, the others from the counter work[colour].
+// (With turns of 8 throughout, a cube of L = 256 kept 256 of 2,432 warps busy: 43 us a sweep, now
+// 13.6; L = 512 70, now 60.)
 // So the groups in flight always form one narrow band that moves through the plane,
 // and the source rows of slices i - 1 and i + 1 are read while they are still in L2
 // (with a fixed grid-stride split the CTAs drift apart over a half-sweep and a row
@@ -267,7 +270,10 @@ __global__ void __launch_bounds__(NT, 2) cubic_half_sweep_kernel(const __grid_co
     uint32_t ups = 0, anti = 0;
     // (i, j, word group) of a lane's group, advanced by 32 groups per step without
     // divisions: step_w groups within a row plus step_r rows, step_r = step_i * L + step_j
-    constexpr int kSteps = 8;
+    const int64_t warps = (int64_t)gridDim.x * (NT / 32);
+    const int64_t turns = ngroups / (64 * warps);
+    const int steps = turns < 1 ? 1 : (turns > 8 ? 8 : (int)turns);
+    int64_t base = 32 * (int64_t)steps * ((int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5));
     const int64_t stride = 32;
     const int64_t step_r = stride / WG;
     const int step_w = (int)(stride - step_r * WG);
@@ -280,11 +286,7 @@ __global__ void __launch_bounds__(NT, 2) cubic_half_sweep_kernel(const __grid_co
     const int64_t step_off = step_r * Wl;
     int64_t row = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) work[colour ^ 1] = 0ull;
-    for (;;) {
-        unsigned long long taken = 0ull;
-        if (lane == 0) taken = atomicAdd(work + colour, 32ull * kSteps);
-        const int64_t base = (int64_t)__shfl_sync(0xffffffffu, taken, 0);
-        if (base >= ngroups) break;
+    while (base < ngroups) {
         {
             const int64_t r0 = (base + lane) / WG;
             wg = (int)(base + lane - r0 * WG);
@@ -294,7 +296,7 @@ __global__ void __launch_bounds__(NT, 2) cubic_half_sweep_kernel(const __grid_co
         }
         // every lane runs every step (the votes and the queue need the whole warp); a
         // lane past the end works on group 0 and keeps nothing
-        for (int s = 0; s < kSteps; ++s) {
+        for (int s = 0; s < steps; ++s) {
             const int64_t g0 = base + 32 * s;
             if (g0 >= ngroups) break;
             const bool valid = g0 + lane < ngroups;
@@ -317,8 +319,8 @@ __global__ void __launch_bounds__(NT, 2) cubic_half_sweep_kernel(const __grid_co
     #pragma unroll
                 for (int k = 0; k < G; ++k) t[k] = trow[k];
             }
-            // q0 = r * (L/8) + 8w = 8 * (row + w) with L/8 = 8W; it is a multiple of 8 * G,
-            // so the group's calls q0 .. q0 + 8G - 1 share q's high word
+            // q0 = r * (L/8) + 8w = 8 * (row + w) with L/8 = 8W; the group's calls
+            // q0 .. q0 + 8G - 1 share q's high word (cubic_words_per_group)
             const uint64_t q0 = 8ull * (uint64_t)(vrow + w);
             const PhiloxWordConsts pc =
                 q_small ? pc_all : philox_consts(d.key, (uint32_t)(q0 >> 32), sweep, (uint32_t)colour);
@@ -384,6 +386,9 @@ __global__ void __launch_bounds__(NT, 2) cubic_half_sweep_kernel(const __grid_co
                 ++i;
             }
         }
+        unsigned long long taken = 0ull;
+        if (lane == 0) taken = atomicAdd(work + colour, 32ull * (unsigned)steps);
+        base = 32 * (int64_t)steps * warps + (int64_t)__shfl_sync(0xffffffffu, taken, 0);
     }
     if (qn > 0) {
         __syncwarp();

@@ -19,8 +19,9 @@
 // another: a tile of a lattice of several tiles carries `halo` extra rows above and below its
 // own, enough for the whole chunk (one row on each side goes stale per half-sweep), reads
 // them from a copy of the planes that no CTA of the launch writes, and writes its own rows
-// to the other copy.
+// to the other copy.  Small cubes go the same way, with slices in the place of rows.
 #include <algorithm>
+#include <type_traits>
 
 #include "ising_internal.cuh"
 #include "philox.cuh"
@@ -218,11 +219,11 @@ __device__ __forceinline__ void draw_step(DrawState& w, const DrawLattice& d, in
     }
 }
 
-// Opens the (M, E) entry of a sweep of an L x L lattice to which several tiles will add their counts.
-__device__ __forceinline__ void open_entry(int64_t* hist, uint32_t sweep, int64_t L)
+// Opens the (M, E) entry of a sweep of N sites in dim dimensions to which several tiles will add their counts.
+__device__ __forceinline__ void open_entry(int64_t* hist, uint32_t sweep, int64_t N, int dim = 2)
 {
-    hist[2 * (int64_t)sweep] = -L * L;
-    hist[2 * (int64_t)sweep + 1] = -2 * L * L;
+    hist[2 * (int64_t)sweep] = -N;
+    hist[2 * (int64_t)sweep + 1] = -dim * N;
 }
 
 // The thresholds' bits as masks, for the drains; formed by one warp of the CTA.
@@ -265,7 +266,7 @@ __device__ void draw_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, u
         if (item >= items) break;
         const int hs = item / per, first = (item - hs * per) * ITEM;
         if (d.tiles > 1 && (hs & 1) == 0 && first == 0 && lane == 0)
-            open_entry(d.hist, sweep0 + (uint32_t)(hs >> 1), d.L);
+            open_entry(d.hist, sweep0 + (uint32_t)(hs >> 1), (int64_t)d.L * d.L);
         draw_step<G, ITEM>(w, one, 0, hs, first, K2, K4, lattice, bits);
     }
     while (w.qn > 0) {
@@ -342,6 +343,96 @@ __device__ __forceinline__ void count_strip(const uint32_t (&t)[K], const uint32
         ups += __popc(s[k] & keep) + __popc(t[k] & keep);
         anti += __popc(odd & keep) + 2u * __popc((both ^ c0 ^ c1) & keep) +
                 4u * __popc(((both & c0) | (both & c1) | (c0 & c1)) & keep);
+    }
+}
+
+// ---- cubes.  A tile is a run of slices instead of rows: a strip is one word column of K
+// consecutive slices, so the neighbours i - 1 and i + 1 are the strip's own words, and the four in
+// the slice (rows j - 1 and j + 1, and the word's own row) come from shared memory.  The three
+// decisions of a site (U < T_2, T_4, T_6, each implying the ones before) are two bits: x = U < T_4,
+// y = U < (x ? T_6 : T_2).
+
+struct CubeStripAt {
+    int t, above, below, left, right, north, south;
+    bool odd;   // of an odd row j: the horizontal neighbours' side is the other one
+    int row;    // its first slice in the tile
+};
+
+template <int K>
+__device__ __forceinline__ CubeStripAt cube_strip_at(const AheadLattice& d, int t)
+{
+    CubeStripAt p;
+    const int S = d.W, R = d.row_words, ty = t / S, tx = t - ty * S, j = tx / R, w = tx - j * R;
+    const bool whole = d.tiles == 1;
+    p.t = t;
+    p.row = ty * K;
+    p.above = ty > 0 ? (K - 1) * kStrips + t - S : (whole ? (K - 1) * kStrips + (d.groups - 1) * S + tx : t);
+    p.below = ty + 1 < d.groups ? t + S : (whole ? tx : t);
+    p.right = w + 1 == R ? t - w : t + 1;
+    p.left = w == 0 ? t + R - 1 : t - 1;
+    p.north = j == 0 ? t + (d.L - 1) * R : t - R;
+    p.south = j + 1 == d.L ? t - (d.L - 1) * R : t + R;
+    p.odd = (j & 1) != 0;
+    return p;
+}
+
+// The neighbour count of one word of a strip (bits b0, b1, b2 of the number of +1 neighbours, 0..6).
+// COLOUR, k: the word's horizontal neighbour is to the right iff k + COLOUR + j is odd.
+template <int COLOUR>
+__device__ __forceinline__ void cube_count(const uint32_t* plane, const CubeStripAt& p, int k, uint32_t up, uint32_t dn,
+                                           uint32_t same, uint32_t& b0, uint32_t& b1, uint32_t& b2)
+{
+    const uint32_t no = plane[p.north + k * kStrips], so = plane[p.south + k * kStrips];
+    const bool right = (((k + COLOUR) & 1) != 0) != p.odd;
+    const uint32_t side = plane[(right ? p.right : p.left) + k * kStrips];
+    const uint32_t hz = __funnelshift_r(right ? same : side, right ? side : same, right ? 1 : 31);
+    const uint32_t s1 = up ^ dn ^ no, c1 = (up & dn) | (no & (up | dn));
+    const uint32_t s2 = so ^ same ^ hz, c2 = (so & same) | (hz & (so | same));
+    const uint32_t c3 = s1 & s2;
+    b0 = s1 ^ s2;
+    b1 = c1 ^ c2 ^ c3;
+    b2 = (c1 & c2) | (c3 & (c1 | c2));
+}
+
+// One colour's half of a sweep for a strip: t its target words, s its source words (in `plane`), m
+// the masks at mp, K words `stride` bytes apart.
+template <int K, int COLOUR>
+__device__ __forceinline__ void update_cube_strip(uint32_t (&t)[K], const uint32_t (&s)[K], const uint32_t* plane,
+                                                  const CubeStripAt& p, const unsigned char* mp, int stride)
+{
+    const uint32_t above = plane[p.above], below = plane[p.below];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        uint32_t b0, b1, b2;
+        cube_count<COLOUR>(plane, p, k, k == 0 ? above : s[k - 1], k == K - 1 ? below : s[k + 1], s[k], b0, b1, b2);
+        const uint2 m = *reinterpret_cast<const uint2*>(mp + k * stride);
+        // n anti-aligned neighbours: c or 6 - c of the c that are +1.  n < 3: c > 3 for a +1, c < 3
+        // for a -1; n odd iff c is; n = 2 rather than 0 iff b1 differs from the spin.
+        const uint32_t h = b2 | (b1 & b0);
+        const uint32_t low = (t[k] & b2) | (~t[k] & ~h);
+        const uint32_t z = b1 ^ t[k];
+        const uint32_t even = (m.x & m.y) | (z & (m.x | m.y));  // n = 2: U < T_2 = x | y; n = 0: U < T_6 = x & y
+        const uint32_t acc = (b0 & m.x) | (~b0 & even);         // n = 1: U < T_4 = x
+        t[k] ^= ~low | acc;
+    }
+}
+
+// Up spins of both colours and anti-aligned bonds of slices lo .. hi - 1 of a strip, from its white
+// words t.
+template <int K>
+__device__ __forceinline__ void count_cube_strip(const uint32_t (&t)[K], const uint32_t (&s)[K], const uint32_t* plane,
+                                                 const CubeStripAt& p, int lo, int hi, uint32_t& ups, uint32_t& anti)
+{
+    const uint32_t above = plane[p.above], below = plane[p.below];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        uint32_t b0, b1, b2;
+        cube_count<1>(plane, p, k, k == 0 ? above : s[k - 1], k == K - 1 ? below : s[k + 1], s[k], b0, b1, b2);
+        const uint32_t keep = k >= lo && k < hi ? ~0u : 0u;
+        // bits of n = 6 - c for a +1, c for a -1
+        const uint32_t n1 = (t[k] & ~(b1 ^ b0)) | (~t[k] & b1), n2 = (t[k] & ~(b2 | (b1 & b0))) | (~t[k] & b2);
+        ups += __popc(s[k] & keep) + __popc(t[k] & keep);
+        anti += __popc(b0 & keep) + 2u * __popc(n1 & keep) + 4u * __popc(n2 & keep);
     }
 }
 
@@ -446,15 +537,15 @@ __device__ __forceinline__ StripNeighbours<K> load_neighbours(const uint32_t* pl
     return nb;
 }
 
-template <int K>
-__device__ __forceinline__ void load_strip(const uint32_t* plane, const StripAt& p, uint32_t (&v)[K])
+template <int K, typename At>
+__device__ __forceinline__ void load_strip(const uint32_t* plane, const At& p, uint32_t (&v)[K])
 {
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = plane[p.t + k * kStrips];
 }
 
-template <int K>
-__device__ __forceinline__ void store_strip(uint32_t* plane, const StripAt& p, const uint32_t (&v)[K])
+template <int K, typename At>
+__device__ __forceinline__ void store_strip(uint32_t* plane, const At& p, const uint32_t (&v)[K])
 {
 #pragma unroll
     for (int k = 0; k < K; ++k) plane[p.t + k * kStrips] = v[k];
@@ -469,10 +560,10 @@ __device__ __forceinline__ void store_strip(uint32_t* plane, const StripAt& p, c
 //    barriers that end the sweep and the next black half-sweep (the black plane has a second
 //    buffer for that);
 //  - a lane of the last warp keeps the ring of masks filled (fetch_masks).
-template <int K>
+template <int K, bool CUBE = false>
 __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile, SharedAhead& sh)
 {
-    const int W = d.W, L = d.L, active = d.groups * W;
+    const int W = d.W, L = d.L, active = d.groups * W;  // (of a cube, W: a slice's words)
     const int threads = (active + 31) & ~31, part = threadIdx.x / kStrips, tid = threadIdx.x % kStrips;
     const bool fetcher = part == 2;
     if (tid >= threads && !fetcher) return;
@@ -486,7 +577,13 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
         fence_mbarrier_init();
     }
     const bool on = tid < active;
-    const StripAt p = strip_at<K>(d, on ? tid : active - 1);  // a lane past the end follows the last one and keeps nothing
+    // a lane past the end follows the last one and keeps nothing
+    const std::conditional_t<CUBE, CubeStripAt, StripAt> p = [&] {
+        if constexpr (CUBE)
+            return cube_strip_at<K>(d, on ? tid : active - 1);
+        else
+            return strip_at<K>(d, on ? tid : active - 1);
+    }();
     const int column = p.t % W;
     // own rows of the strip: k with lo <= k < hi
     const bool whole = d.tiles == 1;
@@ -522,6 +619,17 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
             mp += a.half_bytes;
         };
         auto one_sweep = [&](uint32_t* black) {
+            if constexpr (CUBE) {
+                update_cube_strip<K, 0>(b, w, sh.planes[2], p, mp, W * 8);
+                mp += a.half_bytes;
+                if (on) store_strip<K>(black, p, b);
+                tile_barrier<kBarBlack>(2 * threads);
+                update_cube_strip<K, 1>(w, b, black, p, mp, W * 8);
+                mp += a.half_bytes;
+                if (on) store_strip<K>(sh.planes[2], p, w);
+                tile_barrier<kBarWhite>(2 * threads);
+                return;
+            } else {
             uint2 m[K];
             {
                 const StripNeighbours<K> nb = load_neighbours<K, 0>(sh.planes[2], p, w);
@@ -536,6 +644,7 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
                 update_strip<K>(w, b, nb, m);
                 if (on) store_strip<K>(sh.planes[2], p, w);
                 tile_barrier<kBarWhite>(2 * threads);
+            }
             }
         };
         const int per_slot = st.alone ? n : a.sps;
@@ -584,17 +693,22 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
             tile_barrier<kBarWhite>(2 * threads);
             const uint32_t* black = sh.planes[s & 1];
             load_strip<K>(sh.planes[2], p, w);
-            load_strip<K>(black, p, b);
-            const StripNeighbours<K> nb = load_neighbours<K, 1>(black, p, b);
+            // of what the next black half-sweep's end allows to be overwritten, this was all
             if (s + 1 < n) tile_arrive<kBarBlack>(2 * threads);
+            load_strip<K>(black, p, b);
             uint32_t ups = 0, anti = 0;
+            if constexpr (CUBE) {
+                count_cube_strip<K>(w, b, black, p, lo, hi, ups, anti);
+            } else {
+            const StripNeighbours<K> nb = load_neighbours<K, 1>(black, p, b);
             if (whole) {
                 count_strip<K>(w, b, nb, 0, K, ups, anti);
                 if (!on) ups = anti = 0u;
             } else {
                 count_strip<K>(w, b, nb, lo, hi, ups, anti);
             }
-            // a lane has at most 64 K <= 1024 up spins and 128 K <= 2048 bonds: a warp's sums fit
+            }
+            // a lane has at most 64 K <= 1024 up spins and 128 K <= 2048 bonds (a cube's 192 K): a warp's sums fit
             // 16 bits for strips of up to 8 rows
             uint32_t u, v;
             if (K <= 8) {
@@ -615,13 +729,13 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
     }
     tile_barrier<kBarTile>(everyone);
     if (part == 1) {
-        const int64_t N = (int64_t)L * L;
+        const int64_t N = CUBE ? (int64_t)L * L * L : (int64_t)L * L;
         for (int s = tid; s < n; s += threads) {
             int64_t* entry = d.hist + 2 * (int64_t)(st.upd_sweep + (uint32_t)s);
             const int64_t M = 2 * (int64_t)sh.sums[2 * s], E = 2 * (int64_t)sh.sums[2 * s + 1];
             if (whole) {
                 entry[0] = M - N;
-                entry[1] = E - 2 * N;
+                entry[1] = E - (CUBE ? 3 : 2) * N;
             } else {
                 atomicAdd(reinterpret_cast<unsigned long long*>(entry), (unsigned long long)M);
                 atomicAdd(reinterpret_cast<unsigned long long*>(entry + 1), (unsigned long long)E);
@@ -637,8 +751,8 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
     tile_barrier<kBarTile>(everyone);
 }
 
-// K: rows of a thread's strip.
-template <int K>
+// K: rows (slices of a cube) of a thread's strip.
+template <int K, bool CUBE = false>
 __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ AheadLattice d, const AheadStep st)
 {
     extern __shared__ __align__(16) unsigned char smem_ahead[];
@@ -648,7 +762,7 @@ __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ A
     if (warp == 0) form_bits(d, sh, lane);
     __syncthreads();
     grid_wait();
-    if (st.alone) {
+    if (!CUBE && st.alone) {
         // a short run of a lattice of one tile: this CTA draws the masks it needs itself, into
         // the ring's slots
         int next = warp - kWarps;
@@ -657,7 +771,7 @@ __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ A
         __syncthreads();
     }
     if (st.upd_n > 0)
-        for (int tile = (int)blockIdx.x; tile < d.tiles; tile += (int)gridDim.x) update_tile<K>(d, st, tile, sh);
+        for (int tile = (int)blockIdx.x; tile < d.tiles; tile += (int)gridDim.x) update_tile<K, CUBE>(d, st, tile, sh);
     if (st.fill >= 0) {
         // the first launch of a call: the copy of the planes that the first update reads
         const size_t total = 2 * (size_t)d.words;
@@ -670,9 +784,127 @@ __global__ void __launch_bounds__(kNT, 1) ahead_kernel(const __grid_constant__ A
         d.ticket[st.gen_buf ^ 1] = 0;
         if (st.gen_n == 0) d.ticket[st.gen_buf] = 0;
     }
-    if (st.gen_n > 0)
+    if (CUBE && st.gen_n > 0)
+        draw_cube_chunk(d, st.gen_sweep, st.gen_n, d.masks[st.gen_buf], sh, warp, lane,
+                        [&] { return lane == 0 ? atomicAdd(&d.ticket[st.gen_buf], 1) : 0; });
+    if (!CUBE && st.gen_n > 0)
         draw_chunk<4, kItemWords>(d, st.gen_sweep, st.gen_n, d.masks[st.gen_buf], sh, warp, lane,
                                   [&] { return lane == 0 ? atomicAdd(&d.ticket[st.gen_buf], 1) : 0; });
+}
+
+// ---- drawing for cubes: the same with three thresholds and the two-bit decisions.  An entry of the
+// queue is (undecided against T_2, T_4, T_6; below each so far; word; half-sweep << 3 | next call)
+// in the room of a 2D queue, checked after every word.
+constexpr int kCubeQueueWords = 64;
+static_assert(kCubeQueueWords * 32 <= (int)sizeof(DrawQueue), "a cube's queue fits");
+
+__device__ __forceinline__ uint2 cube_decisions(uint32_t lt2, uint32_t lt4, uint32_t lt6)
+{
+    return make_uint2(lt4, (lt4 & lt6) | (~lt4 & lt2));
+}
+
+__device__ __forceinline__ void drain_cube_draws(const AheadLattice& d, uint32_t sweep0, uint2* masks, uint4* q, int& qn,
+                                                 int n, int lane)
+{
+    uint4 e = make_uint4(0u, 0u, 0u, 0u), f = make_uint4(0u, 0u, 0u, 2u);
+    if (lane < n) {
+        e = q[2 * (qn - n + lane)];
+        f = q[2 * (qn - n + lane) + 1];
+    }
+    qn -= n;
+    __syncwarp();  // entries read before any goes back
+    const uint32_t c = f.w & 7u, hs = f.w >> 3;
+    const PhiloxWordConsts pc = philox_consts(d.key, 0u, sweep0 + (hs >> 1), hs & 1u);
+    const uint32_t base[1] = {8u * f.z ^ pc.x0k};
+    uint32_t o[1][4];
+    philox_calls<1>(base, c, pc, d.key, o);
+    uint32_t l2 = 0u, l4 = 0u, l6 = 0u, e2 = e.x, e4 = e.y, e6 = e.z;
+    const uint32_t t2 = d.t2 << (4u * c), t4 = d.t4 << (4u * c), t6 = d.t6 << (4u * c);
+#pragma unroll
+    for (int m = 3; m >= 0; --m) {
+        compare_plane(o[0][m], plane_mask(t2, m), l2, e2);
+        compare_plane(o[0][m], plane_mask(t4, m), l4, e4);
+        compare_plane(o[0][m], plane_mask(t6, m), l6, e6);
+    }
+    uint32_t lt2 = e.w | (e.x & l2), lt4 = f.x | (e.y & l4), lt6 = f.y | (e.z & l6);
+    if (c == 7u) {  // U equal to min(T, 2^32 - 1): below only if T = 2^32
+        lt2 |= e2 & d.all2;
+        lt4 |= e4 & d.all4;
+        lt6 |= e6 & d.all6;
+    }
+    const bool pend = (e2 | e4 | e6) != 0u && c < 7u;
+    if (lane < n && !pend) masks[(size_t)hs * d.words + f.z] = cube_decisions(lt2, lt4, lt6);
+    const uint32_t bal = __ballot_sync(0xffffffffu, pend);
+    if (pend) {
+        const int slot = qn + __popc(bal & ((1u << lane) - 1u));
+        q[2 * slot] = make_uint4(e2, e4, e6, lt2);
+        q[2 * slot + 1] = make_uint4(lt4, lt6, f.z, f.w + 1u);
+    }
+    qn += __popc(bal);
+}
+
+// A warp's part of drawing a chunk of a cube, 64 words a step (a plane's words are a multiple).
+template <typename Take>
+__device__ void draw_cube_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, uint2* masks, SharedAhead& sh,
+                                int warp, int lane, Take take)
+{
+    constexpr int G = 2;
+    uint4* q = reinterpret_cast<uint4*>(&sh.queue[warp]);
+    int qn = 0;
+    const int per = d.words / (32 * G), items = 2 * sweeps * per;
+    for (;;) {
+        const int item = __shfl_sync(0xffffffffu, take(), 0);
+        if (item >= items) break;
+        const int hs = item / per, word0 = (item - hs * per) * 32 * G + lane;
+        if (d.tiles > 1 && (hs & 1) == 0 && item == hs * per && lane == 0)
+            open_entry(d.hist, sweep0 + (uint32_t)(hs >> 1), (int64_t)d.L * d.L * d.L, 3);
+        const PhiloxWordConsts pc = philox_consts(d.key, 0u, sweep0 + (uint32_t)(hs >> 1), (uint32_t)(hs & 1));
+        uint32_t base[G], lt2[G], lt4[G], lt6[G], eq2[G], eq4[G], eq6[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            base[j] = 8u * (uint32_t)(word0 + 32 * j) ^ pc.x0k;
+            lt2[j] = lt4[j] = lt6[j] = 0u;
+            eq2[j] = eq4[j] = eq6[j] = ~0u;
+        }
+#pragma unroll
+        for (int c = 1; c >= 0; --c) {
+            uint32_t o[G][4];
+            philox_calls<G>(base, (uint32_t)c, pc, d.key, o);
+#pragma unroll
+            for (int m = 3; m >= 0; --m) {
+                const uint32_t K2 = plane_mask(d.t2, 4 * c + m), K4 = plane_mask(d.t4, 4 * c + m),
+                               K6 = plane_mask(d.t6, 4 * c + m);
+#pragma unroll
+                for (int j = 0; j < G; ++j) {
+                    compare_plane(o[j][m], K2, lt2[j], eq2[j]);
+                    compare_plane(o[j][m], K4, lt4[j], eq4[j]);
+                    compare_plane(o[j][m], K6, lt6[j], eq6[j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < G; ++j) {
+            const int word = word0 + 32 * j;
+            const bool pend = (eq2[j] | eq4[j] | eq6[j]) != 0u;
+            if (!pend) masks[(size_t)hs * d.words + word] = cube_decisions(lt2[j], lt4[j], lt6[j]);
+            const uint32_t bal = __ballot_sync(0xffffffffu, pend);
+            if (pend) {
+                const int slot = qn + __popc(bal & ((1u << lane) - 1u));
+                q[2 * slot] = make_uint4(eq2[j], eq4[j], eq6[j], lt2[j]);
+                q[2 * slot + 1] = make_uint4(lt4[j], lt6[j], (uint32_t)word, (uint32_t)hs << 3 | 2u);
+            }
+            qn += __popc(bal);
+            while (qn >= 32) {
+                __syncwarp();  // pushes visible to the draining lanes
+                drain_cube_draws(d, sweep0, masks, q, qn, 32, lane);
+            }
+        }
+    }
+    while (qn > 0) {
+        __syncwarp();
+        drain_cube_draws(d, sweep0, masks, q, qn, min(qn, 32), lane);
+    }
+    __syncwarp();
 }
 
 // ---- batches: the same for many lattices of a batch, in common launches.  The geometry of each
@@ -838,7 +1070,8 @@ __global__ void __launch_bounds__(kNT, 1) ahead_batch_kernel(const __grid_consta
         if (st.gen_off + (hs >> 1) >= sweeps_of(ld, st.total)) continue;
         const int first = (r - step_start[l]) * kItemWords;
         const DrawLattice d = lattice(l);
-        if (!batch_whole(ld.W, b.dense) && (hs & 1) == 0 && first == 0 && lane == 0) open_entry(ld.hist, d.sweep0 + (uint32_t)(hs >> 1), ld.L);
+        if (!batch_whole(ld.W, b.dense) && (hs & 1) == 0 && first == 0 && lane == 0) 
+            open_entry(ld.hist, d.sweep0 + (uint32_t)(hs >> 1), (int64_t)ld.L * ld.L);
         uint32_t K2[8], K4[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -853,10 +1086,10 @@ __global__ void __launch_bounds__(kNT, 1) ahead_batch_kernel(const __grid_consta
     }
 }
 
-template <int K>
+template <int K, bool CUBE = false>
 cudaError_t launch_k(const AheadLattice& d, const AheadStep& st, int grid, cudaStream_t s)
 {
-    return launch_following(ahead_kernel<K>, dim3(grid), dim3(kNT), sizeof(SharedAhead), s, d, st);
+    return launch_following(ahead_kernel<K, CUBE>, dim3(grid), dim3(kNT), sizeof(SharedAhead), s, d, st);
 }
 
 cudaError_t launch_step(const AheadLattice& d, const AheadStep& st, cudaStream_t s)
@@ -864,6 +1097,7 @@ cudaError_t launch_step(const AheadLattice& d, const AheadStep& st, cudaStream_t
     const int64_t items = 2 * (int64_t)st.gen_n * ((d.words + kItemWords - 1) / kItemWords);
     const int64_t want = (st.upd_n > 0 ? d.tiles : 0) + (items + kWarps - 1) / kWarps;
     const int64_t grid = std::min<int64_t>(sm_count(), std::max<int64_t>(want, 1));
+    if (d.cube) return launch_k<16, true>(d, st, (int)grid, s);
     switch (d.strip) {
     case 2:
         return launch_k<2>(d, st, (int)grid, s);
@@ -972,9 +1206,37 @@ AheadPlan ahead_plan(int64_t L)
     return p;
 }
 
+// Cubes whose slice (L * L/64 words) is one thread's word each: L = 64 in one tile, L = 128 in tiles
+// of 16 slices.
+AheadPlan ahead_plan3(int64_t L)
+{
+    AheadPlan p;
+    if (L != 64 && L != 128) return p;
+    const int S = (int)(L * (L / 64));
+    const int64_t per_sweep = L * S * 2 * (int64_t)sizeof(uint2);
+    p.cube = 1;
+    p.strip = kMaxStrip;
+    p.groups = kStrips / S;
+    if (L == 64) {
+        p.rows = (int)L;
+        p.halo = 0;
+        p.tiles = 1;
+        p.chunk = (int)((8ll << 20) / per_sweep);
+    } else {
+        p.chunk = 3;
+        p.halo = 2 * p.chunk;
+        p.rows = p.groups * p.strip - 2 * p.halo;
+        p.tiles = (int)((L + p.rows - 1) / p.rows);
+        p.copy_bytes = 2 * 2 * L * S * (int64_t)sizeof(uint32_t);
+    }
+    p.mask_bytes = per_sweep * p.chunk;
+    return p;
+}
+
 cudaError_t ahead_configure(const AheadPlan& p)
 {
-    const void* k = p.strip == 2   ? (const void*)ahead_kernel<2>
+    const void* k = p.cube         ? (const void*)ahead_kernel<16, true>
+                    : p.strip == 2 ? (const void*)ahead_kernel<2>
                     : p.strip == 4 ? (const void*)ahead_kernel<4>
                     : p.strip == 8 ? (const void*)ahead_kernel<8>
                                    : (const void*)ahead_kernel<16>;
@@ -985,7 +1247,7 @@ cudaError_t ahead_configure(const AheadPlan& p)
 // the drawing alone.
 bool ahead_alone(const AheadLattice& d, int64_t n)
 {
-    return d.tiles == 1 && n <= kWarps && 2 * n * ((d.words + 31) / 32) <= 2 * kWarps;
+    return !d.cube && d.tiles == 1 && n <= kWarps && 2 * n * ((d.words + 31) / 32) <= 2 * kWarps;
 }
 
 cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s)

@@ -125,3 +125,18 @@ def test_batch_matches_tiled(Ls):
         b.close()
     for ((ma, ea), la), ((mt, et), lt) in zip(*out):
         assert np.array_equal(ma, mt) and np.array_equal(ea, et) and np.array_equal(la, lt)
+
+
+# L = 64 in one tile (chunks of 64 and 128 sweeps), L = 128 in tiles of 4 own slices (chunks of 3)
+@pytest.mark.parametrize("L,runs", [(64, [20, 70, 150, 1]), (128, [17, 3, 2])])
+@pytest.mark.parametrize("beta", [0.0, 0.2216546, 200.0])
+def test_cube_matches_oracle(L, runs, beta):
+    n = sum(runs)
+    lat = ising.Lattice3D(L, beta, 7 + L, ising.HOT)
+    for r in runs:
+        lat.sweep(r)
+    ref, M, E, _ = oracle.run3d((L, L, L), beta, 7 + L, oracle.HOT, n)
+    m, e = lat.history(0, n)
+    assert np.array_equal(m, M) and np.array_equal(e, E)
+    assert np.array_equal(lat.get_lattice(), ref)
+    lat.close()
