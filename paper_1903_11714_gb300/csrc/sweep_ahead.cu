@@ -156,10 +156,10 @@ __device__ __forceinline__ void drain_draws(DrawState& w, int n, Lattice lattice
 // calls (planes 7..4, then 3..0) for every word, side by side: they decide about 78 % of the
 // words for all 32 sites and both thresholds; the others finish from the warp's queue, a word per
 // lane.  K2, K4: the thresholds' bits of the first eight planes as masks.
-template <int G, bool FULL, typename Lattice, typename Bits>
+template <int G, bool FULL, typename Lattice, typename Bits, typename Then>
 __device__ __forceinline__ void draw_words(DrawState& w, const DrawLattice& d, int index, const PhiloxWordConsts& pc, int hs,
                                            int word0, const uint32_t (&K2)[8], const uint32_t (&K4)[8], Lattice lattice,
-                                           Bits bits)
+                                           Bits bits, Then then)
 {
     uint32_t base[G], lt2[G], lt4[G], eq2[G], eq4[G];
 #pragma unroll
@@ -180,6 +180,7 @@ __device__ __forceinline__ void draw_words(DrawState& w, const DrawLattice& d, i
                 compare_plane(o[j][m], K4[4 * c + m], lt4[j], eq4[j]);
             }
     }
+    then();
     uint2* const out = d.masks + (size_t)hs * d.words + word0 + w.lane;
 #pragma unroll
     for (int j = 0; j < G; ++j) {
@@ -203,19 +204,19 @@ __device__ __forceinline__ void draw_words(DrawState& w, const DrawLattice& d, i
 }
 
 // One drawing step: words first .. first + ITEM - 1 (as far as they exist) of half-sweep hs.
-template <int G, int ITEM, typename Lattice, typename Bits>
+template <int G, int ITEM, typename Lattice, typename Bits, typename Then>
 __device__ __forceinline__ void draw_step(DrawState& w, const DrawLattice& d, int index, int hs, int first,
-                                          const uint32_t (&K2)[8], const uint32_t (&K4)[8], Lattice lattice, Bits bits)
+                                          const uint32_t (&K2)[8], const uint32_t (&K4)[8], Lattice lattice, Bits bits, Then then)
 {
     const PhiloxWordConsts pc = philox_consts(d.key, 0u, d.sweep0 + (uint32_t)(hs >> 1), (uint32_t)(hs & 1));
     if (first + ITEM <= d.words) {
-#pragma unroll 1
-        for (int k = 0; k < ITEM; k += 32 * G)
-            draw_words<G, true>(w, d, index, pc, hs, first + k, K2, K4, lattice, bits);
+        static_assert(ITEM == 32 * G, "a step is one group");
+        draw_words<G, true>(w, d, index, pc, hs, first, K2, K4, lattice, bits, then);
     } else {
+        then();
 #pragma unroll 1
         for (int word0 = first; word0 < d.words; word0 += 32)
-            draw_words<1, false>(w, d, index, pc, hs, word0, K2, K4, lattice, bits);
+            draw_words<1, false>(w, d, index, pc, hs, word0, K2, K4, lattice, bits, [] {});
     }
 }
 
@@ -267,7 +268,7 @@ __device__ void draw_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, u
         const int hs = item / per, first = (item - hs * per) * ITEM;
         if (d.tiles > 1 && (hs & 1) == 0 && first == 0 && lane == 0)
             open_entry(d.hist, sweep0 + (uint32_t)(hs >> 1), (int64_t)d.L * d.L);
-        draw_step<G, ITEM>(w, one, 0, hs, first, K2, K4, lattice, bits);
+        draw_step<G, ITEM>(w, one, 0, hs, first, K2, K4, lattice, bits, [] {});
     }
     while (w.qn > 0) {
         __syncwarp();
@@ -276,10 +277,16 @@ __device__ void draw_chunk(const AheadLattice& d, uint32_t sweep0, int sweeps, u
     __syncwarp();
 }
 
-// Named barriers of a tile's `threads` threads: of those that hold strips and those that count,
-// at the end of a black half-sweep (the counting ones only arrive) and of a white one; and of
-// all parts of the CTA.
-constexpr int kBarBlack = 1, kBarWhite = 2, kBarTile = 3;
+// Named barriers: of all parts of a tile, and, one pair for even and one for odd sweeps, of the
+// threads that hold strips and those that count the sweep, at the end of its white half (kBarWhite
+// + parity) and of the next sweep's black half (kBarBlack + the next one's parity; the counting
+// threads only arrive).
+constexpr int kBarTile = 1, kBarBlack = 2, kBarWhite = 4;
+
+__device__ __forceinline__ void tile_barrier(int id, int threads)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
 template <int ID>
 __device__ __forceinline__ void tile_barrier(int threads)
@@ -287,10 +294,9 @@ __device__ __forceinline__ void tile_barrier(int threads)
     asm volatile("bar.sync %0, %1;" ::"n"(ID), "r"(threads) : "memory");
 }
 
-template <int ID>
-__device__ __forceinline__ void tile_arrive(int threads)
+__device__ __forceinline__ void tile_arrive(int id, int threads)
 {
-    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "r"(threads) : "memory");
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
@@ -558,17 +564,23 @@ __device__ __forceinline__ void store_strip(uint32_t* plane, const At& p, const 
 //  - as many threads of the second group count the own rows' (M, E) of a sweep while the
 //    first already runs the next one: they take the words from shared memory between the
 //    barriers that end the sweep and the next black half-sweep (the black plane has a second
-//    buffer for that);
+//    buffer for that).  Tiles of at most half the strips have two such groups, a sweep each in
+//    turn, as counting takes longer than updating (L = 128: 300 ns a sweep counted by the
+//    first group, 237 by one group beside it, 180 by two; L = 64: 154);
 //  - a lane of the last warp keeps the ring of masks filled (fetch_masks).
 template <int K, bool CUBE = false>
 __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile, SharedAhead& sh)
 {
     const int W = d.W, L = d.L, active = d.groups * W;  // (of a cube, W: a slice's words)
-    const int threads = (active + 31) & ~31, part = threadIdx.x / kStrips, tid = threadIdx.x % kStrips;
+    const int threads = (active + 31) & ~31, part = threadIdx.x / kStrips;
+    // tiles of at most half the strips are counted by two groups in turn, a sweep each
+    const int turns = threads <= kStrips / 2 ? 2 : 1;
+    const int turn = turns == 2 && part == 1 ? threadIdx.x % kStrips / (kStrips / 2) : 0;
+    const int tid = threadIdx.x % kStrips - turn * (kStrips / 2);
     const bool fetcher = part == 2;
     if (tid >= threads && !fetcher) return;
     const TileAt a = tile_at<K>(d, tile);
-    const int n = st.upd_n, everyone = 2 * threads + 32;
+    const int n = st.upd_n, everyone = (1 + turns) * threads + 32;
     if (threadIdx.x == 0 && !st.alone) {
         for (int k = 0; k < a.slots; ++k) {
             mbar_init(&sh.full[k], 1);
@@ -618,33 +630,34 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
             for (int k = 0; k < K; ++k) m[k] = *reinterpret_cast<const uint2*>(mp + k * (W * 8));
             mp += a.half_bytes;
         };
-        auto one_sweep = [&](uint32_t* black) {
+        auto one_sweep = [&](auto which) {
+            constexpr int parity = decltype(which)::value;
+            uint32_t* const black = sh.planes[parity];
             if constexpr (CUBE) {
                 update_cube_strip<K, 0>(b, w, sh.planes[2], p, mp, W * 8);
                 mp += a.half_bytes;
                 if (on) store_strip<K>(black, p, b);
-                tile_barrier<kBarBlack>(2 * threads);
+                tile_barrier<kBarBlack + parity>(2 * threads);
                 update_cube_strip<K, 1>(w, b, black, p, mp, W * 8);
                 mp += a.half_bytes;
                 if (on) store_strip<K>(sh.planes[2], p, w);
-                tile_barrier<kBarWhite>(2 * threads);
-                return;
+                tile_barrier<kBarWhite + parity>(2 * threads);
             } else {
-            uint2 m[K];
-            {
-                const StripNeighbours<K> nb = load_neighbours<K, 0>(sh.planes[2], p, w);
-                load_masks(m);
-                update_strip<K>(b, w, nb, m);
-                if (on) store_strip<K>(black, p, b);
-                tile_barrier<kBarBlack>(2 * threads);
-            }
-            {
-                const StripNeighbours<K> nb = load_neighbours<K, 1>(black, p, b);
-                load_masks(m);
-                update_strip<K>(w, b, nb, m);
-                if (on) store_strip<K>(sh.planes[2], p, w);
-                tile_barrier<kBarWhite>(2 * threads);
-            }
+                uint2 m[K];
+                {
+                    const StripNeighbours<K> nb = load_neighbours<K, 0>(sh.planes[2], p, w);
+                    load_masks(m);
+                    update_strip<K>(b, w, nb, m);
+                    if (on) store_strip<K>(black, p, b);
+                    tile_barrier<kBarBlack + parity>(2 * threads);
+                }
+                {
+                    const StripNeighbours<K> nb = load_neighbours<K, 1>(black, p, b);
+                    load_masks(m);
+                    update_strip<K>(w, b, nb, m);
+                    if (on) store_strip<K>(sh.planes[2], p, w);
+                    tile_barrier<kBarWhite + parity>(2 * threads);
+                }
             }
         };
         const int per_slot = st.alone ? n : a.sps;
@@ -656,16 +669,16 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
             }
             int left = min(per_slot, n - s);
             if (odd) {
-                one_sweep(sh.planes[1]);
+                one_sweep(std::integral_constant<int, 1>());
                 odd = 0;
                 --left;
             }
             for (; left >= 2; left -= 2) {
-                one_sweep(sh.planes[0]);
-                one_sweep(sh.planes[1]);
+                one_sweep(std::integral_constant<int, 0>());
+                one_sweep(std::integral_constant<int, 1>());
             }
             if (left) {
-                one_sweep(sh.planes[0]);
+                one_sweep(std::integral_constant<int, 0>());
                 odd = 1;
             }
             if (!st.alone) {
@@ -688,28 +701,32 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
                 dst[d.words + at] = w[k];
             }
     } else if (part == 1) {
-        tile_arrive<kBarBlack>(2 * threads);
-        for (int s = 0; s < n; ++s) {
-            tile_barrier<kBarWhite>(2 * threads);
+        const bool strips = whole || (d.halo % K == 0 && d.rows % K == 0 && L % d.rows % K == 0);  // own rows are whole strips
+        // (for the first black half-sweep, which has no sweep before it)
+        if (turn == turns - 1) tile_arrive(kBarBlack, 2 * threads);
+        for (int s = turn; s < n; s += turns) {
+            tile_barrier(kBarWhite + (s & 1), 2 * threads);
             const uint32_t* black = sh.planes[s & 1];
             load_strip<K>(sh.planes[2], p, w);
             // of what the next black half-sweep's end allows to be overwritten, this was all
-            if (s + 1 < n) tile_arrive<kBarBlack>(2 * threads);
+            // (arriving after the other loads is still faster by 5 % at L = 128)
+            if (CUBE && s + 1 < n) tile_arrive(kBarBlack + ((s + 1) & 1), 2 * threads);
             load_strip<K>(black, p, b);
             uint32_t ups = 0, anti = 0;
             if constexpr (CUBE) {
                 count_cube_strip<K>(w, b, black, p, lo, hi, ups, anti);
             } else {
-            const StripNeighbours<K> nb = load_neighbours<K, 1>(black, p, b);
-            if (whole) {
-                count_strip<K>(w, b, nb, 0, K, ups, anti);
-                if (!on) ups = anti = 0u;
-            } else {
-                count_strip<K>(w, b, nb, lo, hi, ups, anti);
+                const StripNeighbours<K> nb = load_neighbours<K, 1>(black, p, b);
+                if (s + 1 < n) tile_arrive(kBarBlack + ((s + 1) & 1), 2 * threads);
+                if (strips) {
+                    count_strip<K>(w, b, nb, 0, K, ups, anti);
+                    if (lo >= hi) ups = anti = 0u;
+                } else {
+                    count_strip<K>(w, b, nb, lo, hi, ups, anti);
+                }
             }
-            }
-            // a lane has at most 64 K <= 1024 up spins and 128 K <= 2048 bonds (a cube's 192 K): a warp's sums fit
-            // 16 bits for strips of up to 8 rows
+            // a lane has at most 64 K <= 1024 up spins and 128 K <= 2048 bonds (a cube's 192 K): a
+            // warp's sums fit 16 bits for strips of up to 8 rows
             uint32_t u, v;
             if (K <= 8) {
                 const uint32_t both = __reduce_add_sync(0xffffffffu, ups | (anti << 16));
@@ -730,7 +747,7 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
     tile_barrier<kBarTile>(everyone);
     if (part == 1) {
         const int64_t N = CUBE ? (int64_t)L * L * L : (int64_t)L * L;
-        for (int s = tid; s < n; s += threads) {
+        for (int s = turn * threads + tid; s < n; s += turns * threads) {
             int64_t* entry = d.hist + 2 * (int64_t)(st.upd_sweep + (uint32_t)s);
             const int64_t M = 2 * (int64_t)sh.sums[2 * s], E = 2 * (int64_t)sh.sums[2 * s + 1];
             if (whole) {
@@ -1059,15 +1076,18 @@ __global__ void __launch_bounds__(kNT, 1) ahead_batch_kernel(const __grid_consta
         b4 = make_uint4(plane_mask(t4, 0), plane_mask(t4, 1), plane_mask(t4, 2), plane_mask(t4, 3));
     };
     const int per = step_start[b.count], items = 2 * st.gen_n * per;
+    auto take = [&] { return lane == 0 ? atomicAdd(&b.ticket[st.gen_buf], 1) : 0; };
+    int taken = take();
     for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(&b.ticket[st.gen_buf], 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
+        const int item = __shfl_sync(0xffffffffu, taken, 0);
         if (item >= items) break;
         const int hs = item / per, r = item - hs * per;
         const int l = find_entry(step_start, b.count, r);
         const LatticeDesc& ld = b.desc[l];
-        if (st.gen_off + (hs >> 1) >= sweeps_of(ld, st.total)) continue;
+        if (st.gen_off + (hs >> 1) >= sweeps_of(ld, st.total)) {
+            taken = take();
+            continue;
+        }
         const int first = (r - step_start[l]) * kItemWords;
         const DrawLattice d = lattice(l);
         if (!batch_whole(ld.W, b.dense) && (hs & 1) == 0 && first == 0 && lane == 0) 
@@ -1078,7 +1098,7 @@ __global__ void __launch_bounds__(kNT, 1) ahead_batch_kernel(const __grid_consta
             K2[k] = plane_mask(d.t2, k);
             K4[k] = plane_mask(d.t4, k);
         }
-        draw_step<4, kItemWords>(w, d, l, hs, first, K2, K4, lattice, bits);
+        draw_step<4, kItemWords>(w, d, l, hs, first, K2, K4, lattice, bits, [&] { taken = take(); });
     }
     while (w.qn > 0) {
         __syncwarp();
