@@ -702,10 +702,16 @@ __device__ void update_tile(const AheadLattice& d, const AheadStep& st, int tile
             }
     } else if (part == 1) {
         const bool strips = whole || (d.halo % K == 0 && d.rows % K == 0 && L % d.rows % K == 0);  // own rows are whole strips
+        // a warp whose strips are all halo rows only keeps the barriers' count
+        const bool any_own = __any_sync(0xffffffffu, lo < hi);
         // (for the first black half-sweep, which has no sweep before it)
         if (turn == turns - 1) tile_arrive(kBarBlack, 2 * threads);
         for (int s = turn; s < n; s += turns) {
             tile_barrier(kBarWhite + (s & 1), 2 * threads);
+            if (!any_own) {
+                if (s + 1 < n) tile_arrive(kBarBlack + ((s + 1) & 1), 2 * threads);
+                continue;
+            }
             const uint32_t* black = sh.planes[s & 1];
             load_strip<K>(sh.planes[2], p, w);
             // of what the next black half-sweep's end allows to be overwritten, this was all
@@ -1208,15 +1214,18 @@ AheadPlan ahead_plan(int64_t L)
         // Several tiles.  A launch costs about 4 us beyond its half-sweeps, which asks for long
         // chunks; their halo rows are updated (and their masks fetched) by two tiles, which
         // asks for short ones, the more so the more the drawing of the own rows' masks takes.
-        // us a sweep: L = 256: 0.59 in one tile, 0.51 with strips of 2 and chunks of 24; 320:
-        // 0.81 / 0.55 (20); 512: 1.03, 0.77, 0.69 with strips of 4 and chunks of 8, 16, 24; 1,024:
-        // 1.05 (8), 0.88 (12), strips of 8 1.08 (20); 1,344: strips of 8 1.19 (16), of 16 2.0;
-        // 2,048: strips of 8 2.16 (8), of 16 1.89 (20); 4,096: 6.95 (4), 6.63 (8), 7.06 (10);
-        // 8,192: 26.7 (2), 25.9 (3), 26.6 (4)
+        // us a sweep: L = 256: 0.59 in one tile, 0.48 and 0.46 with strips of 2 and chunks of 24 and
+        // 28; 320: 0.81 / 0.54 (20); 512: strips of 4 0.65 (24), 0.63 (28), of 2 0.64 (14); 1,024: strips
+        // of 4 0.93 (10), 0.88 (12), 1.13 (14), of 8 1.08 (20); 1,344: strips of 8 1.19 (16), of
+        // 16 2.0; 2,048: strips of 8 2.15 (8), of 16 1.71 (16), 1.77 (20); 4,096: 6.70 (6), 6.42 (8),
+        // 6.80 (10); 8,192: 26.7 (2), 25.9 (3), 26.8 (4)
         p.strip = W <= 6 ? 2 : (W <= 16 ? 4 : (W <= 28 ? 8 : 16));
         p.groups = kStrips / W;
         const int held = p.groups * p.strip;  // rows a CTA holds
-        p.chunk = W <= 28 ? std::min(32, held * 3 / 16) : (W <= 32 ? held * 5 / 32 : (W <= 64 ? held / 8 : held * 3 / 32));
+        p.chunk = W <= 8    ? std::min(32, held * 7 / 32)
+                  : W <= 28 ? held * 3 / 16
+                  : W <= 64 ? held / 8
+                            : held * 3 / 32;
         p.halo = 2 * p.chunk;
         p.rows = held - 2 * p.halo;
         p.tiles = (int)((L + p.rows - 1) / p.rows);
