@@ -176,9 +176,19 @@ int default_tile_rows(int64_t L, int threads = 256)
     return tr;
 }
 
+// Time of a half-sweep of one lattice in tiles of tr rows, in words a CTA updates one after the
+// other: the rounds of tiles over `slots` resident CTAs, and a tile's words in whole steps of the
+// CTA (a group of up to four adjacent words a thread) plus its own cost, about a word a thread.
+int64_t rounds_cost(int64_t L, int tr, int threads, int64_t slots)
+{
+    const int64_t W = L / 64, step = threads * (W % 4 == 0 ? 4 : (W % 2 == 0 ? 2 : 1));
+    return (L / tr + slots - 1) / slots * ((W * tr + step - 1) / step * step + threads);
+}
+
 // Tile height for a lattice swept on its own (the single-lattice instance, two
 // CTAs per SM): the built-in height, lowered so that small lattices are cut into
-// enough tiles to spread over the persistent grid instead of a few large ones.
+// enough tiles to spread over the persistent grid instead of a few large ones; beyond
+// L = 8,192 the cheapest by rounds_cost.
 int single_tile_rows(int64_t L)
 {
     const int grid = 2 * sm_count();
@@ -186,7 +196,13 @@ int single_tile_rows(int64_t L)
     while (tr < kMaxTileRows && L / tr > grid) tr *= 2;
     tr = std::min(tr, default_tile_rows(L));
     while (tr > 2 && !tile_rows_ok(L, tr)) tr >>= 1;
-    return tile_rows_ok(L, tr) ? tr : default_tile_rows(L);
+    if (!tile_rows_ok(L, tr)) return default_tile_rows(L);
+    if (L <= 8192) return tr;
+    for (int t = 4; t <= kMaxTileRows; t *= 2)
+        if (tile_rows_ok(L, t) && t * (L / 64) <= 6144 && L / t >= grid &&
+            rounds_cost(L, t, 256, grid) < rounds_cost(L, tr, 256, grid))
+            tr = t;
+    return tr;
 }
 
 // CTA size and tile height of a lattice swept on its own.  Sides of at least 16,384
@@ -194,7 +210,11 @@ int single_tile_rows(int64_t L)
 // so that each of its 16 warps still handles about 512 words of a tile: the per-tile
 // costs (the last partial drain of each warp's queue, the stage handoff) are then a
 // smaller share than with two 256-thread CTAs of 4,096-word tiles (+2 % at L = 65,536;
-// 512-thread CTAs with 4,096-word tiles lose 6 %).  Other sides: 256 threads and
+// 512-thread CTAs with 4,096-word tiles lose 6 %).  The height is the
+// cheapest by rounds_cost: 8,192 words leave the last round of the SMs nearly empty at L =
+// 16,384 (512 tiles in 3.4 rounds), and 5,120 words are two and a half steps of the CTA.
+// flips/ns, tallest of up to 8,192 words / cheapest: L = 16,384 3,569 / 3,760; 17,408 2,734 / 3,340;
+// 20,480 3,377 / 3,741; 40,960 3,667 / 4,549.  Other sides: 256 threads and
 // single_tile_rows.
 void single_config(int64_t L, int* tile_rows, int* threads)
 {
@@ -202,10 +222,13 @@ void single_config(int64_t L, int* tile_rows, int* threads)
     *tile_rows = single_tile_rows(L);
     const int64_t W = L / 64;
     if (L < 16384 || !whole_rows_ok(L)) return;
+    const int64_t sms = sm_count();
     int best = 0;
     for (int tr = 2; tr <= kMaxTileRows; tr *= 2)
-        if (tile_rows_ok(L, tr) && W * tr <= 8192 && L / tr >= 2 * sm_count()) best = tr;
-    if (best && W * best >= 4096) {
+        if (tile_rows_ok(L, tr) && W * tr >= 2048 && W * tr <= 12288 && L / tr >= 2 * sms &&
+            (!best || rounds_cost(L, tr, 512, sms) <= rounds_cost(L, best, 512, sms)))
+            best = tr;
+    if (best) {
         *threads = 512;
         *tile_rows = best;
     }

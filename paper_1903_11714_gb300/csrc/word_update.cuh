@@ -97,15 +97,14 @@ __device__ __forceinline__ void classify_word(uint32_t t, uint32_t up, uint32_t 
     const uint32_t s0 = au ^ ad, c0 = au & ad;
     const uint32_t s1 = as ^ ah, c1 = as & ah;
     const uint32_t b0 = s0 ^ s1, cc = s0 & s1;
-    const uint32_t b1 = c0 ^ c1 ^ cc;
-    const uint32_t b2 = c0 & c1;
-    // n >= 2 (h <= 0): always; n == 1 (h = 2): U < T2; n == 0 (h = 4): U < T4
-    const uint32_t always = b1 | b2;
-    const uint32_t h2 = b0 & ~always, h4 = ~b0 & ~always;
-    f = always | (h2 & all2) | (h4 & all4);
-    und = (h2 & ~(all2 | zero2)) | (h4 & ~(all4 | zero4));
+    // n >= 2 (h <= 0): always -- two in one pair (c0, c1) or one in each (cc, never with them);
+    // n == 1 (h = 2): U < T2; n == 0 (h = 4): U < T4
+    const uint32_t always = c0 | c1 | cc;
+    f = always | (b0 & all2) | (~b0 & all4);
+    und = ~always & ((b0 & ~(all2 | zero2)) | (~b0 & ~(all4 | zero4)));
     sel = b0;
-    anti0 = __popc(b0) - 2u * __popc(b1) - 4u * __popc(b2);
+    // popc(b1) + 2 popc(b2) = popc(c0) + popc(c1) + popc(cc)
+    anti0 = __popc(b0) - 2u * __popc(always) - 2u * __popc(c0 & c1);
 }
 
 template <int G, bool COUNT>
