@@ -576,6 +576,18 @@ int ensure_hist(ising_t h, int64_t need)
 uint32_t thr32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : (uint32_t)T; }
 uint32_t all32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : 0u; }
 
+// cudaMalloc for a workspace that a sweep call may need for the first time while another thread
+// captures a graph on a stream of its own: such a capture forbids the call in its strictest mode
+// unless this thread relaxes its own.
+cudaError_t malloc_relaxed(char** p, size_t bytes)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMalloc(p, bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
+}
+
 // The sweep with its random numbers drawn ahead: the lattice's plan and constants.
 int setup_ahead(ising_t h)
 {
@@ -625,7 +637,7 @@ bool ahead_ready(ising_t h, int64_t n)
         return false;
     }
     char* ws = nullptr;
-    if (cudaMalloc(&ws, (size_t)(2 * p.mask_bytes + p.copy_bytes + 256)) != cudaSuccess ||
+    if (malloc_relaxed(&ws, (size_t)(2 * p.mask_bytes + p.copy_bytes + 256)) != cudaSuccess ||
         cudaMemsetAsync(ws, 0, 256, h->stream) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(ws);
@@ -1475,6 +1487,7 @@ int update_cluster(ising_batch_t b)
 //    32 uneven lattices of 2.1e7 sites 21.4 us, 9.5 drawn ahead); they cross at 1.2e8 sites;
 //  - cluster-resident: 3,000 + 1,420 for each word a thread holds of a plane (64 x 1,024: 16
 //    words, 25.7 us; 8 x 1,024: 8.7, drawn ahead 3.7; 256 x 128: 4.9 and 2.6).
+constexpr int64_t kAheadMaxBatchSites = 130000000;  // a workspace of 0.6 GB
 void update_ahead(ising_batch_t b)
 {
     b->ahead_wanted = false;
@@ -1488,7 +1501,7 @@ void update_ahead(ising_batch_t b)
         sites += s.L * s.L;
         longest = std::max(longest, s.L);
     }
-    if (longest == 0) return;
+    if (longest == 0 || sites > kAheadMaxBatchSites) return;
     const double sms = sm_count(), S = (double)sites, drawn_ahead = 350.0 + S / (2300.0 * sms / 152.0);
     double other = (S + 2.5e7) / (2690.0 * sms / 152.0);
     const ClusterPlan& c = b->eng.cluster;
@@ -1542,7 +1555,7 @@ int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
         // most twice the last one)
         char* ws = nullptr;
         const int64_t bytes = b->ahead_ws ? need + need / 2 : need;
-        if (cudaMalloc(&ws, (size_t)bytes) != cudaSuccess) {
+        if (malloc_relaxed(&ws, (size_t)bytes) != cudaSuccess) {
             cudaGetLastError();
             b->ahead_refused = true;
             return ISING_OK;

@@ -87,13 +87,14 @@ int64_t stage_bytes(int64_t L, int tr)
     return (stage_words((int32_t)W, tr, (int32_t)halo_rows(W)) * 4 + 15) / 16 * 16;
 }
 
-// Tile height for tiles of at most `words` words (4 rows at least).
-constexpr int64_t kTileWords = 4096, kLeastTileWords = 256;
-int tile_rows_for(int64_t L, int64_t words)
+// About 4,096 words a tile.  (Halving the tiles of a call with fewer than two for each SM gained 2 %
+// for sides that are multiples of 256 and lost 18 % for others, whose tiles carry four halo rows
+// on either side.)
+int tile_rows_for(int64_t L)
 {
     const int64_t W = L / 64;
     int tr = 64;
-    while (tr > 4 && (int64_t)tr * W > words) tr >>= 1;
+    while (tr > 4 && (int64_t)tr * W > 4096) tr >>= 1;
     while (tr > 4 && (L % tr != 0 || stage_bytes(L, tr) > kNoAllocStageCap)) tr >>= 1;
     return tr;
 }
@@ -150,7 +151,7 @@ extern "C" int ising_sweep_packed_noalloc(int32_t count, uint32_t* const* black,
         if (!black[k] || !white[k] || !me[k]) return set_error(ISING_EINVAL, "null plane or output pointer");
         uint64_t T[2];
         if (ising_thresholds(beta[k], T) != ISING_OK) return set_error(ISING_EINVAL, "beta must be finite and >= 0");
-        const int tr = tile_rows_for(L[k], kTileWords);
+        const int tr = tile_rows_for(L[k]);
         if (stage_bytes(L[k], tr) > kNoAllocStageCap)
             return set_error(ISING_EINVAL, "L too large for a shared-memory tile: L <= 163840 (L % 256 == 0) or L <= 102336");
         LatticeDesc& d = p.desc[k];
@@ -190,20 +191,6 @@ extern "C" int ising_sweep_packed_noalloc(int32_t count, uint32_t* const* black,
     DeviceState* st = nullptr;
     int rc = device_setup(dev, &st);
     if (rc) return rc;
-    // a call of few or small lattices holds fewer tiles of 4,096 words than the GPU has SMs, and a
-    // half-sweep takes as long as its tile: halve the tiles until every SM has two of them (256
-    // words at least: a thread's group is four)
-    for (int64_t words = kTileWords / 2; words >= kLeastTileWords && tiles < 2 * (int64_t)st->sms; words /= 2) {
-        tiles = 0;
-        stage = 16;
-        for (int k = 0; k < count; ++k) {
-            const int tr = tile_rows_for(L[k], words);
-            p.desc[k].tile_rows = tr;
-            tiles += L[k] / tr;
-            stage = stage_bytes(L[k], tr) > stage ? stage_bytes(L[k], tr) : stage;
-            p.tile_start[k + 1] = (int32_t)tiles;
-        }
-    }
     // persistent grid: as many CTAs as fit with this call's stage size
     const size_t smem = (size_t)packed_smem_header_bytes(kNoAllocThreads) + 2 * (size_t)stage;
     int per_sm = 0;
