@@ -42,6 +42,39 @@ def test_ahead_matches_oracle(L, beta):
     lat.close()
 
 
+# runs of one handle that alternate between the launch that draws its own masks, the tiled kernel
+# (until 16 sweeps have been asked for) and the masks drawn ahead
+@pytest.mark.parametrize("L,runs", [(64, [1, 9, 2, 3, 8, 1, 20]), (128, [2, 3, 1, 5, 2, 9, 1]), (256, [1, 9, 3, 5, 1])])
+def test_routes_alternate(L, runs):
+    lat = ising.Lattice(L, 0.43, 31, ising.HOT)
+    check(lat, L, 0.43, 31, ising.HOT, runs)
+    lat.close()
+
+
+# a run captured into a caller's graph, before (9 sweeps) and after (20) the workspace exists
+@pytest.mark.parametrize("L", [64, 192, 512])
+@pytest.mark.parametrize("before", [9, 20])
+def test_captured_run(L, before):
+    import torch
+
+    stream = torch.cuda.Stream()
+    lat = ising.Lattice(L, 0.43, 32, ising.HOT, stream=stream)
+    lat.sweep(before)
+    lat.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+        lat.sweep(17)
+    with torch.cuda.stream(stream):
+        g.replay()
+    lat.sweep(4)
+    ref, M, E, _ = oracle.run(L, 0.43, 32, ising.HOT, before + 21)
+    m, e = lat.history(0, before + 21)
+    assert np.array_equal(m, M) and np.array_equal(e, E)
+    assert np.array_equal(lat.get_lattice(), ref)
+    del g
+    lat.close()
+
+
 def test_long_runs_cross_chunks():
     # L = 128: chunks of 64, 1024 and the rest; L = 256: chunks of 24
     for L, runs in ((128, [3, 1200, 40]), (256, [600, 9])):
