@@ -1518,15 +1518,21 @@ void update_ahead(ising_batch_t b)
 }
 
 // Whether a run of n sweeps goes that way: the workspace and the tables are made ready by the
-// first run that needs them, once the batch has been asked for 16 sweeps in all (before
-// that, where memory is short and on a stream that is being captured: the tiled or the
-// cluster-resident kernel, as otherwise).
+// first run that needs them, once the batch has been asked for 16 sweeps in all.  Before that,
+// where memory is short and on a stream that is being captured: the tiled or the
+// cluster-resident kernel, as otherwise (the launches here carry the batch's tables by value, so
+// a graph of them would not follow a batch that changes between its replays).
 constexpr int64_t kAheadMinBatchSweeps = 16;
 int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
 {
     *ready = false;
     b->ahead_asked = std::min<int64_t>(b->ahead_asked + n, kAheadMinBatchSweeps);
     if (!b->ahead_wanted || b->ahead_refused || b->ahead_asked < kAheadMinBatchSweeps) return ISING_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return ISING_OK;
+    }
     if (b->ahead_tables) {
         *ready = true;
         return ISING_OK;
@@ -1543,11 +1549,6 @@ int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
     const int64_t W = words[b->count], table_bytes = 256 + (3 * ((int64_t)ahead_batch_max_count() + 1) * 4 + 255) / 256 * 256;
     const int64_t mask_bytes = (W * 2 * a.chunk * (int64_t)sizeof(uint2) + 255) / 256 * 256;
     const int64_t need = table_bytes + 2 * mask_bytes + W * 16;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return ISING_OK;
-    }
     if (need > b->ahead_ws_bytes) {
         CK(ahead_batch_configure());
         // half as much again for lattices yet to come; the outgrown workspace stays until the

@@ -75,6 +75,31 @@ def test_captured_run(L, before):
     lat.close()
 
 
+def test_captured_batch_run_follows_the_batch():
+    # a graph of a batch's run, replayed after another lattice has joined, sweeps it too
+    import torch
+
+    stream = torch.cuda.Stream()
+    b = ising.Batch(4, 320, 1 << 22, 0, stream)
+    first = b.add(320, 0.41, 7, ising.HOT, 100)
+    b.add(64, 0.39, 9, ising.HOT, 100)
+    b.run(20)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+        b.run(17)
+    second = b.add(128, 0.44, 8, ising.HOT, 100)
+    with torch.cuda.stream(stream):
+        g.replay()
+    b.run(5)
+    for k, L, beta, seed, n in ((first, 320, 0.41, 7, 42), (second, 128, 0.44, 8, 22)):
+        ref, M, E, _ = oracle.run(L, beta, seed, ising.HOT, n)
+        m, e = b.history(k)
+        assert np.array_equal(m, M) and np.array_equal(e, E)
+        assert np.array_equal(b.get_lattice(k), ref)
+    del g
+    b.close()
+
+
 def test_long_runs_cross_chunks():
     # L = 128: chunks of 64, 1024 and the rest; L = 256: chunks of 24
     for L, runs in ((128, [3, 1200, 40]), (256, [600, 9])):
