@@ -200,6 +200,8 @@ __global__ void __launch_bounds__(kThreads, 2) int8_half_sweep_seg64_kernel(cons
     // at most 2^27 strips (L <= 131,072)
     const int idx = (int)(blockIdx.x * kThreads + threadIdx.x);
     const bool valid = idx < G * (int)(L / rows);  // the votes need the whole warp: a lane past the end keeps nothing
+    // a lane past the end counts no words of its own, but does count those that a drain hands it
+    const bool counts = valid && d.colour == 1;
     const int strip = valid ? idx / G : 0, g = valid ? idx - strip * G : 0;
     const int64_t i0 = (int64_t)strip * rows;
     grid_wait();
@@ -237,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 2) int8_half_sweep_seg64_kernel(cons
             uint32_t anti0;
             classify_word(t[k], up, dn, same[k], hz, d.all2, d.all4, zero2, zero4, f[k], und[k], sel[k], anti0);
             if (!valid) und[k] = 0u;
-            if (d.colour == 1) anti += anti0;
+            if (counts) anti += anti0;
             ql[k] = 8u * (uint32_t)((i + k) * G + g);
         }
         // calls 0-1 (planes 0-7) without a test: nearly every word needs both
@@ -251,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 2) int8_half_sweep_seg64_kernel(cons
                 for (int m = 0; m < 4; ++m)
                     if ((f[k] >> (8 * m)) & 0xFFu) row[m] = raw[k][m];
             }
-            if (d.colour == 1) {
+            if (counts) {
                 // the word as decided so far; the drain adds the rest
                 negs += __popc(same[k]) + __popc(t[k] ^ f[k]);
                 anti += 4u * __popc(f[k]) - 2u * __popc(f[k] & sel[k]);
@@ -279,7 +281,6 @@ __global__ void __launch_bounds__(kThreads, 2) int8_half_sweep_seg64_kernel(cons
     }
     if (d.colour == 1) {
         // a drained word's counts may be negative for the lane that drained it
-        if (!valid) negs = anti = 0u;
         block_add_pair(-2ll * (int32_t)negs, 2ll * (int32_t)anti, d.hist_slot);
     }
 }
