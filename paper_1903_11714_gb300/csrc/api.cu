@@ -417,10 +417,10 @@ struct Engine {
 
     int check_status()
     {
-        PinnedBlock blk;
-        if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
-        CK(launch_report(nullptr, nullptr, 0, 0, d_status, blk.words(), stream));
-        CK(cudaStreamSynchronize(stream));
+        ReportBlock blk;
+        if (!blk.ok()) return cuda_fail(blk.error, "report block");
+        CK(launch_report(nullptr, nullptr, 0, 0, d_status, blk.target(), stream));
+        CK(blk.fetch(sizeof(int64_t), stream));
         return judge(blk.words()[0]);
     }
 
@@ -474,7 +474,7 @@ struct Arena : FreeList {
 void ising::set_last_error(const char* msg) { t_error = msg; }
 
 namespace {
-// A handle's or batch's share in the page-locked blocks (readback.cu).
+// A handle's or batch's share in the report blocks (report_block.h).
 struct ReadbackUser {
     ReadbackUser() { readback_user(1); }
     ~ReadbackUser() { readback_user(-1); }
@@ -750,11 +750,11 @@ int read_status(ising_t h)
 // The handle's status word on the device (its sweeps may give up a bounded wait), or null.
 const int* status_word(ising_t h) { return h->kernel != ISING_INT8 ? h->eng.d_status : nullptr; }
 
-// Waits for the stream and judges the status a report put into st.
-int await_report(ising_t h, const int64_t* st)
+// Waits for a report of n 64-bit words and judges its status.
+int await_report(ising_t h, ReportBlock& blk, int64_t n)
 {
-    CK(cudaStreamSynchronize(h->stream));
-    return h->kernel != ISING_INT8 ? h->eng.judge(*st) : ISING_OK;
+    CK(blk.fetch(sizeof(int64_t) * (size_t)n, h->stream));
+    return h->kernel != ISING_INT8 ? h->eng.judge(blk.words()[0]) : ISING_OK;
 }
 
 // Copies the lattice to host int8 through a bounded device staging buffer.
@@ -1124,11 +1124,11 @@ int ising_observables(ising_t h, int64_t* M, int64_t* E, int64_t* sweeps_done)
 {
     int rc = check_handle(h);
     if (rc) return rc;
-    PinnedBlock blk;
-    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
+    ReportBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "report block");
     const int64_t* src = h->sweeps_done ? h->hist + 2 * (h->sweeps_done - 1) : h->d_me0;
-    CK(launch_report(nullptr, src, 0, 1, status_word(h), blk.words(), h->stream));
-    rc = await_report(h, blk.words());
+    CK(launch_report(nullptr, src, 0, 1, status_word(h), blk.target(), h->stream));
+    rc = await_report(h, blk, 4);
     if (rc) return rc;
     const int64_t* me = blk.words() + 2;
     if (M) *M = me[0];
@@ -1146,11 +1146,11 @@ int ising_history(ising_t h, int64_t first, int64_t count, int64_t* M, int64_t* 
                     (long long)(first + count), (long long)h->sweeps_done);
     std::vector<int64_t> buf;
     const int64_t* e;
-    PinnedBlock blk;
-    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
-    if (count <= PinnedBlock::kEntries) {
-        CK(launch_report(nullptr, h->hist, first, count, status_word(h), blk.words(), h->stream));
-        rc = await_report(h, blk.words());
+    ReportBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "report block");
+    if (count <= ReportBlock::kEntries) {
+        CK(launch_report(nullptr, h->hist, first, count, status_word(h), blk.target(), h->stream));
+        rc = await_report(h, blk, 2 + 2 * count);
         e = blk.words() + 2;
     } else {
         buf.resize(2 * (size_t)count);
@@ -1173,16 +1173,15 @@ int ising_moments_ex(ising_t h, int64_t burn_in, double out[6], uint64_t sums[11
     if (rc) return rc;
     if (!out) return fail(ISING_EINVAL, "null output");
     if (burn_in < 0 || burn_in >= h->sweeps_done) return fail(ISING_EINVAL, "no samples after burn-in");
-    PinnedBlock blk;
-    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
-    double* m = reinterpret_cast<double*>(blk.words() + 2);
-    uint64_t* t = reinterpret_cast<uint64_t*>(blk.words() + 8);
-    CK(launch_moments(nullptr, h->hist, burn_in, h->sweeps_done - burn_in, site_count(h), m, t, status_word(h),
-                      blk.words(), h->stream));
-    rc = await_report(h, blk.words());
+    ReportBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "report block");
+    int64_t* t = blk.target();
+    CK(launch_moments(nullptr, h->hist, burn_in, h->sweeps_done - burn_in, site_count(h), reinterpret_cast<double*>(t + 2),
+                      reinterpret_cast<uint64_t*>(t + 8), status_word(h), t, h->stream));
+    rc = await_report(h, blk, 19);
     if (rc) return rc;
-    memcpy(out, m, 6 * sizeof(double));
-    if (sums) memcpy(sums, t, 11 * sizeof(uint64_t));
+    memcpy(out, blk.words() + 2, 6 * sizeof(double));
+    if (sums) memcpy(sums, blk.words() + 8, 11 * sizeof(uint64_t));
     return ISING_OK;
 }
 
@@ -1265,16 +1264,15 @@ int ising_get_planes(ising_t h, uint32_t* black, uint32_t* white)
     if (rc) return rc;
     if (h->kernel == ISING_INT8) return fail(ISING_EINVAL, "not a packed handle");
     const size_t bytes = sizeof(uint32_t) * (size_t)plane_words(h);
-    if (2 * bytes + 16 <= (size_t)PinnedBlock::kBytes) {
-        PinnedBlock blk;
-        if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
-        uint32_t* w = static_cast<uint32_t*>(blk.p);
-        w[0] = w[1] = 0u;
-        CK(launch_report_words(h->planes, 2 * plane_words(h), status_word(h), w, h->stream));
-        rc = await_report(h, blk.words());
+    if (2 * bytes + 16 <= (size_t)ReportBlock::kBytes) {
+        ReportBlock blk;
+        if (!blk.ok()) return cuda_fail(blk.error, "report block");
+        CK(launch_report_words(h->planes, 2 * plane_words(h), status_word(h), blk.target(), h->stream));
+        rc = await_report(h, blk, 2 + plane_words(h));
         if (rc) return rc;
-        if (black) memcpy(black, w + 4, bytes);
-        if (white) memcpy(white, w + 4 + plane_words(h), bytes);
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(blk.words() + 2);
+        if (black) memcpy(black, w, bytes);
+        if (white) memcpy(white, w + plane_words(h), bytes);
         return ISING_OK;
     }
     if (black) CK(cudaMemcpyAsync(black, h->planes, bytes, cudaMemcpyDeviceToHost, h->stream));
@@ -1640,17 +1638,17 @@ int check_batch(ising_batch_t b, int32_t idx)
 
 // One report of slot idx: its sweep count, and count history entries from `first` on (left out
 // where they lie beyond that).
-int batch_report(ising_batch_t b, int32_t idx, int64_t first, int64_t count, const PinnedBlock& blk)
+int batch_report(ising_batch_t b, int32_t idx, int64_t first, int64_t count, ReportBlock& blk)
 {
-    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
-    CK(launch_report(b->eng.d_desc + idx, nullptr, first, count, b->eng.d_status, blk.words(), b->stream));
-    CK(cudaStreamSynchronize(b->stream));
+    if (!blk.ok()) return cuda_fail(blk.error, "report block");
+    CK(launch_report(b->eng.d_desc + idx, nullptr, first, count, b->eng.d_status, blk.target(), b->stream));
+    CK(blk.fetch(sizeof(int64_t) * (size_t)(2 + 2 * count), b->stream));
     return b->eng.judge(blk.words()[0]);
 }
 
 int batch_sweeps_done(ising_batch_t b, int32_t idx, int64_t* done)
 {
-    PinnedBlock blk;
+    ReportBlock blk;
     int rc = batch_report(b, idx, 0, 0, blk);
     if (rc) return rc;
     *done = blk.words()[1];
@@ -1957,15 +1955,15 @@ int ising_batch_observables_ex(ising_batch_t b, int32_t idx, int64_t* M, int64_t
 {
     int rc = check_batch(b, idx);
     if (rc) return rc;
-    PinnedBlock blk;
+    ReportBlock blk;
     rc = batch_report(b, idx, kLastEntry, 1, blk);
     if (rc) return rc;
     const int64_t done = blk.words()[1];
     if (done == 0) {
         const auto& d = b->slots[idx].desc;
         CK(launch_packed_observe(d.plane[0], d.plane[1], d.L, b->d_me, b->stream));
-        CK(launch_report(nullptr, b->d_me, 0, 1, nullptr, blk.words(), b->stream));
-        CK(cudaStreamSynchronize(b->stream));
+        CK(launch_report(nullptr, b->d_me, 0, 1, nullptr, blk.target(), b->stream));
+        CK(blk.fetch(4 * sizeof(int64_t), b->stream));
     }
     const int64_t* me = blk.words() + 2;
     if (M) *M = me[0];
@@ -1984,8 +1982,8 @@ int ising_batch_history(ising_batch_t b, int32_t idx, int64_t first, int64_t cou
     int rc = check_batch(b, idx);
     if (rc) return rc;
     // (a negative range asks the device for no entry and is refused below)
-    const bool small = first >= 0 && count >= 0 && count <= PinnedBlock::kEntries;
-    PinnedBlock blk;
+    const bool small = first >= 0 && count >= 0 && count <= ReportBlock::kEntries;
+    ReportBlock blk;
     rc = batch_report(b, idx, small ? first : 0, small ? count : 0, blk);
     if (rc) return rc;
     const int64_t done = blk.words()[1];
@@ -2013,19 +2011,18 @@ int ising_batch_moments(ising_batch_t b, int32_t idx, int64_t burn_in, double ou
     if (rc) return rc;
     if (!out) return fail(ISING_EINVAL, "null output");
     const auto& d = b->slots[idx].desc;
-    PinnedBlock blk;
-    if (!blk.ok()) return cuda_fail(blk.error, "cudaHostAlloc");
-    double* m = reinterpret_cast<double*>(blk.words() + 2);
-    uint64_t* t = reinterpret_cast<uint64_t*>(blk.words() + 8);
+    ReportBlock blk;
+    if (!blk.ok()) return cuda_fail(blk.error, "report block");
+    int64_t* t = blk.target();
     // (a negative burn_in asks for no sample and is refused below)
-    CK(launch_moments(b->eng.d_desc + idx, nullptr, burn_in < 0 ? INT64_MAX : burn_in, 0, (int64_t)d.L * d.L, m, t,
-                      b->eng.d_status, blk.words(), b->stream));
-    CK(cudaStreamSynchronize(b->stream));
+    CK(launch_moments(b->eng.d_desc + idx, nullptr, burn_in < 0 ? INT64_MAX : burn_in, 0, (int64_t)d.L * d.L,
+                      reinterpret_cast<double*>(t + 2), reinterpret_cast<uint64_t*>(t + 8), b->eng.d_status, t, b->stream));
+    CK(blk.fetch(19 * sizeof(int64_t), b->stream));
     rc = b->eng.judge(blk.words()[0]);
     if (rc) return rc;
     if (burn_in < 0 || burn_in >= blk.words()[1]) return fail(ISING_EINVAL, "no samples after burn-in");
-    memcpy(out, m, 6 * sizeof(double));
-    if (sums) memcpy(sums, t, 11 * sizeof(uint64_t));
+    memcpy(out, blk.words() + 2, 6 * sizeof(double));
+    if (sums) memcpy(sums, blk.words() + 8, 11 * sizeof(uint64_t));
     return ISING_OK;
 }
 

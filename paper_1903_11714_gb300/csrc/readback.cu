@@ -4,23 +4,11 @@
 // memory take the driver about 10 us each, and a look at one batch lattice's history was three
 // of them: the histories and moments of 64 lattices took 6.7 ms, now 2.9; one sweep of L = 64
 // with its (M, E) and planes 49 us, now 36.
-//
-// The page-locked blocks are shared by the process: a call takes one for its duration, so two
-// threads never share one; at most kKept wait for the next call, and all are given back when the
-// last handle is freed.
-#include <mutex>
-#include <vector>
-
 #include "ising_internal.cuh"
 #include "readback.h"
 
 namespace ising {
 namespace {
-
-constexpr size_t kKept = 8;
-std::mutex g_mu;
-std::vector<void*> g_free;
-int64_t g_users = 0;
 
 __global__ void report_kernel(const LatticeDesc* desc, const int64_t* hist, int64_t first, int64_t count,
                               const int* status, int64_t* out)
@@ -40,46 +28,13 @@ __global__ void report_words_kernel(const uint32_t* words, int64_t n, const int*
 {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
         out[4 + k] = words[k];
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = status ? (uint32_t)*status : 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        out[0] = status ? (uint32_t)*status : 0u;
+        out[1] = 0u;
+    }
 }
 
 }  // namespace
-
-void readback_user(int change)
-{
-    std::vector<void*> unused;
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        g_users += change;
-        if (g_users == 0) unused.swap(g_free);
-    }
-    for (void* p : unused) cudaFreeHost(p);
-}
-
-PinnedBlock::PinnedBlock()
-{
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (!g_free.empty()) {
-            p = g_free.back();
-            g_free.pop_back();
-        }
-    }
-    if (!p) error = cudaHostAlloc(&p, kBytes, cudaHostAllocPortable | cudaHostAllocMapped);
-}
-
-PinnedBlock::~PinnedBlock()
-{
-    if (!p) return;
-    {
-        std::lock_guard<std::mutex> lock(g_mu);
-        if (g_users > 0 && g_free.size() < kKept) {
-            g_free.push_back(p);
-            return;
-        }
-    }
-    cudaFreeHost(p);
-}
 
 cudaError_t launch_report(const LatticeDesc* desc, const int64_t* hist, int64_t first, int64_t count, const int* status,
                           int64_t* out, cudaStream_t s)
@@ -89,9 +44,10 @@ cudaError_t launch_report(const LatticeDesc* desc, const int64_t* hist, int64_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_report_words(const uint32_t* words, int64_t n, const int* status, uint32_t* out, cudaStream_t s)
+cudaError_t launch_report_words(const uint32_t* words, int64_t n, const int* status, int64_t* out, cudaStream_t s)
 {
-    report_words_kernel<<<(unsigned)((n + 1023) / 1024 + 1), 256, 0, s>>>(words, n, status, out);
+    report_words_kernel<<<(unsigned)((n + 1023) / 1024 + 1), 256, 0, s>>>(words, n, status,
+                                                                         reinterpret_cast<uint32_t*>(out));
     return cudaGetLastError();
 }
 
