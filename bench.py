@@ -538,6 +538,7 @@ def run_cubic(args) -> None:
     clocks = sampler.stop()
     lat.synchronize()
     ms = e0.elapsed_time(e1)
+    launches = lat.last_run()[1]
     lat.close()
     value = steps * N / (ms * 1e6)
     t_launch_s = ms * 1e-3 / (2 * steps)
@@ -551,7 +552,7 @@ def run_cubic(args) -> None:
         "ms_per_step": ms / steps, "higher_is_better": True,
         "config": {**cfg.as_dict(), "l2": "inputs larger than L2 (1 GB planes vs 129 MB L2), no flush"},
         "roofline": roofline,
-        "cpu_baseline": cpu, "gpu_launches": 2 * steps, "clocks": clocks}))
+        "cpu_baseline": cpu, "gpu_launches": launches, "clocks": clocks}))
 
 
 def run_binder3d(args) -> None:
@@ -821,13 +822,11 @@ def main() -> None:
     flips_all = total_over_ranks(float(args.steps * N), dist, "cuda")
     value = flips_all / (ms * 1e6)
 
-    # dominant kernel: the packed half-sweep (2 launches per sweep + 1 counter advance per call)
-    launches = 2 * args.steps + 1
-    # a lattice of L <= 8,192 draws its random numbers ahead in chunks of sweeps: at least one launch
-    # that draws and one that applies, and none of the half-sweep kernel that the counters describe
-    ahead = kernel == ising.PACKED and L <= 8192 and args.warmup + args.steps >= 16
-    if ahead:
-        launches = 2
+    # the kernels that the timed call enqueued, by the library's own count
+    form, launches = lat.last_run()
+    # a lattice of L <= 8,192 draws its random numbers ahead in chunks of sweeps: none of the half-sweep
+    # kernel that the counters describe
+    ahead = form == ising.RUN_AHEAD
     t_launch_s = ms * 1e-3 / (2 * args.steps)
     if kernel == ising.PACKED:
         roofline = kernel_roofline("packed_half_sweep", N / 2, t_launch_s, sm_max, peaks)

@@ -257,6 +257,23 @@ int ising_batch_specialized(ising_batch_t b, int32_t *specialized);
 int ising_batch_set_cluster(ising_batch_t b, int32_t mode);
 int ising_batch_cluster_size(ising_batch_t b, int32_t *cluster_size);
 
+/*
+ * What the last run with n > 0 sweeps was (ising_sweep; ising_batch_run): *form, the kernels
+ * it took, and *launches, how many it enqueued (those inside replayed graphs counted
+ * one by one).  The forms give the same chain bit for bit; which one runs follows from the
+ * sides, the length of the run and the memory to be had.  Either output may be NULL.
+ * Host-only.  Paper: none (it reports the schedule of the Sec. 3.1 sweep).
+ * Errors: EINVAL (null handle).
+ */
+#define ISING_RUN_NONE 0     /* no sweep yet */
+#define ISING_RUN_TILED 1    /* one launch per half-sweep, tiles staged through shared memory */
+#define ISING_RUN_AHEAD 2    /* random numbers drawn ahead of the update, chunks of sweeps per launch */
+#define ISING_RUN_CLUSTER 3  /* batches: lattices resident in thread-block clusters */
+#define ISING_RUN_BYTES 4    /* the int8 kernel */
+#define ISING_RUN_CUBIC 5    /* three dimensions, one launch per half-sweep */
+int ising_last_run(ising_t h, int32_t *form, int64_t *launches);
+int ising_batch_last_run(ising_batch_t b, int32_t *form, int64_t *launches);
+
 /* Releases the handle and its device memory (NULL is a no-op).  Paper: none (resource
  * management of the Sec. 3 lattice). */
 int ising_free(ising_t h);

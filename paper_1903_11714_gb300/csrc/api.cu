@@ -264,6 +264,7 @@ struct Engine {
     ClusterPlan cluster;
     int64_t cluster_L = 0;
     int cluster_count = 0;
+    int64_t launched = 0;      // kernels that the last run enqueued
     bool blocks = false;       // some lattice has column-block tiles (launch the build that handles them)
 
     void allow_blocks()
@@ -362,11 +363,13 @@ struct Engine {
         }
         cudaError_t e = launch_packed_advance(d_desc, d_count, max_count, (int)n, stream);
         if (e != cudaSuccess) return cuda_fail(e, "advance launch");
+        launched = 2 * n + 1;
         return ISING_OK;
     }
 
     int run(int64_t sweeps, int graph_sweeps)
     {
+        launched = 0;
         if (sweeps == 0) return ISING_OK;
         if (cluster.C > 0) {
             // every lattice stays in its cluster's shared memory for up to 4,096 sweeps per
@@ -377,6 +380,7 @@ struct Engine {
                 cudaError_t e = launch_packed_advance(d_desc, d_count, max_count, chunk, stream);
                 if (e != cudaSuccess) return cuda_fail(e, "advance launch");
                 done += chunk;
+                launched += 2;
             }
             return ISING_OK;
         }
@@ -404,6 +408,7 @@ struct Engine {
             it = graphs.emplace(graph_sweeps, ge).first;
         }
         for (int64_t r = 0; r < sweeps / graph_sweeps; ++r) CK(cudaGraphLaunch(it->second, stream));
+        launched = sweeps / graph_sweeps * (2 * graph_sweeps + 1);
         return ISING_OK;
     }
 
@@ -474,6 +479,18 @@ struct Arena : FreeList {
 void ising::set_last_error(const char* msg) { t_error = msg; }
 
 namespace {
+// What the last run was (ising_last_run).
+struct LastRun {
+    int32_t form = ISING_RUN_NONE;
+    int64_t launches = 0;
+    int get(int32_t* form_out, int64_t* launches_out) const
+    {
+        if (form_out) *form_out = form;
+        if (launches_out) *launches_out = launches;
+        return ISING_OK;
+    }
+};
+
 // A handle's or batch's share in the report blocks (report_block.h).
 struct ReadbackUser {
     ReadbackUser() { readback_user(1); }
@@ -484,6 +501,7 @@ struct ReadbackUser {
 // ====================================================================== handles
 struct ising_s {
     ReadbackUser readback;
+    LastRun last;
     int64_t L = 0;
     double beta = 0;
     uint64_t seed = 0;
@@ -513,6 +531,7 @@ struct ising_s {
 
 struct ising_batch_s {
     ReadbackUser readback;
+    LastRun last;
     struct Slot {
         bool used = false;
         int64_t L = 0;
@@ -1079,11 +1098,15 @@ int ising_sweep(ising_t h, int64_t n)
     if (rc) return rc;
     if (ahead_ready(h, n)) {
         h->ahead.hist = h->hist;
-        CK(launch_ahead_sweeps(h->ahead, h->ahead_plan.chunk, (uint32_t)h->sweeps_done, n, h->stream));
+        int64_t launched = 0;
+        CK(launch_ahead_sweeps(h->ahead, h->ahead_plan.chunk, (uint32_t)h->sweeps_done, n, h->stream, &launched));
+        h->last = {ISING_RUN_AHEAD, launched};
     } else if (h->kernel == ISING_PACKED) {
         rc = h->eng.run(n, 0);
         if (rc) return rc;
+        h->last = {ISING_RUN_TILED, h->eng.launched};
     } else if (h->kernel == kKernelCubic) {
+        h->last = {ISING_RUN_CUBIC, 2 * n};
         const CubicDesc d = cubic_desc(h);
         for (int64_t k = 0; k < n; ++k)
             for (int c = 0; c < 2; ++c) {
@@ -1092,6 +1115,7 @@ int ising_sweep(ising_t h, int64_t n)
                 if (e != cudaSuccess) return cuda_fail(e, "3D half-sweep launch");
             }
     } else {
+        h->last = {ISING_RUN_BYTES, 2 * n};
         uint32_t t2, t4, all2, all4;
         LatticeDesc tmp{};
         set_thresholds(tmp, h->T);
@@ -1111,6 +1135,12 @@ int ising_sweep(ising_t h, int64_t n)
     h->sweeps_done += n;
     h->desc.sweep = (uint32_t)h->sweeps_done;
     return ISING_OK;
+}
+
+int ising_last_run(ising_t h, int32_t* form, int64_t* launches)
+{
+    const int rc = check_handle(h);
+    return rc ? rc : h->last.get(form, launches);
 }
 
 int ising_synchronize(ising_t h)
@@ -1877,15 +1907,19 @@ int ising_batch_run(ising_batch_t b, int64_t sweeps, int32_t graph_sweeps)
     if (rc) return rc;
     if (ahead) {
         // in parts whose sweep numbers fit the launch parameters; no graph is needed
+        int64_t launched = 0;
         for (int64_t done = 0; done < sweeps;) {
             const int64_t n = std::min<int64_t>(sweeps - done, 1 << 20);
-            CK(launch_ahead_batch(b->ahead, b->ahead_steps, n, b->stream));
+            CK(launch_ahead_batch(b->ahead, b->ahead_steps, n, b->stream, &launched));
             CK(launch_packed_advance(b->eng.d_desc, b->eng.d_count, b->eng.max_count, (int)n, b->stream));
             done += n;
+            ++launched;
         }
-    } else {
+        b->last = {ISING_RUN_AHEAD, launched};
+    } else if (sweeps > 0) {
         rc = b->eng.run(sweeps, graph_sweeps);
         if (rc) return rc;
+        b->last = {b->eng.cluster.C > 0 ? ISING_RUN_CLUSTER : ISING_RUN_TILED, b->eng.launched};
     }
     if (b->growable)
         for (auto& s : b->slots)
@@ -1929,6 +1963,12 @@ int ising_batch_cluster_size(ising_batch_t b, int32_t* cluster_size)
     if (!b || !cluster_size) return fail(ISING_EINVAL, "null argument");
     *cluster_size = b->eng.cluster.C;
     return ISING_OK;
+}
+
+int ising_batch_last_run(ising_batch_t b, int32_t* form, int64_t* launches)
+{
+    if (!b) return fail(ISING_EINVAL, "null batch");
+    return b->last.get(form, launches);
 }
 
 int ising_batch_specialized(ising_batch_t b, int32_t* specialized)

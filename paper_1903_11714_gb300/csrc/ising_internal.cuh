@@ -116,16 +116,18 @@ int ahead_batch_chunk(int64_t L);               // sweeps of a launch, for the b
 int32_t ahead_batch_tiles(int64_t L, int chunk, int dense);
 int32_t ahead_batch_steps(int64_t L);
 cudaError_t ahead_batch_configure();
-// Enqueues a run of n sweeps; steps: drawing steps of a half-sweep of all lattices.
-cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s);
+// Enqueues a run of n sweeps; steps: drawing steps of a half-sweep of all lattices.  Adds its
+// launches to *launched.
+cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s, int64_t* launched);
 int ahead_max_L();
 AheadPlan ahead_plan(int64_t L);
 AheadPlan ahead_plan3(int64_t L);  // of a cube
 cudaError_t ahead_configure(const AheadPlan& p);
 // Whether n sweeps are one launch of one CTA that draws its own masks (no workspace needed).
 bool ahead_alone(const AheadLattice& d, int64_t n);
-// Enqueues n sweeps, numbered from `sweep` on, in launches of at most `chunk` sweeps.
-cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s);
+// Enqueues n sweeps, numbered from `sweep` on, in launches of at most `chunk` sweeps, added to *launched.
+cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s,
+                                int64_t* launched);
 cudaError_t launch_packed_advance(LatticeDesc* desc, const int32_t* count, int max_count, int steps,
                                   cudaStream_t s);
 // Cluster-resident sweeps (sweep_cluster.cu): lattices of one side L <= cluster_max_L()

@@ -1165,7 +1165,7 @@ cudaError_t ahead_batch_configure()
     return cudaFuncSetAttribute(ahead_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SharedAhead));
 }
 
-cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s)
+cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cudaStream_t s, int64_t* launched)
 {
     // chunk k is drawn by the launch that updates chunk k - 1, as for a single lattice
     int64_t drawn = 0, updated = 0;
@@ -1186,6 +1186,7 @@ cudaError_t launch_ahead_batch(const AheadBatch& b, int64_t steps, int64_t n, cu
         const int grid = (int)std::min<int64_t>(sm_count(), want);
         const cudaError_t e = launch_following(ahead_batch_kernel, dim3(grid), dim3(kNT), sizeof(SharedAhead), s, b, st);
         if (e != cudaSuccess) return e;
+        ++*launched;
         updated += in_flight;
         drawn += next;
         in_flight = next;
@@ -1279,7 +1280,8 @@ bool ahead_alone(const AheadLattice& d, int64_t n)
     return !d.cube && d.tiles == 1 && n <= kWarps && 2 * n * ((d.words + 31) / 32) <= 2 * kWarps;
 }
 
-cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s)
+cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s,
+                                int64_t* launched)
 {
     AheadStep st;
     st.upd_n = st.gen_n = 0;
@@ -1290,6 +1292,7 @@ cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep
         st.alone = 1;
         st.upd_sweep = sweep;
         st.upd_n = (int)n;
+        ++*launched;
         return launch_step(d, st, s);
     }
     // chunk k is drawn into buffer k & 1 by the launch that updates chunk k - 1.  Of a lattice
@@ -1311,6 +1314,7 @@ cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep
         }
         cudaError_t e = launch_step(d, st, s);
         if (e != cudaSuccess) return e;
+        ++*launched;
         updated += in_flight;
         drawn += next;
         in_flight = next;

@@ -68,6 +68,8 @@ _SIGS = {
     "ising_batch_specialized": (ctypes.c_int, [_vp, _P(_i32)]),
     "ising_batch_set_cluster": (ctypes.c_int, [_vp, _i32]),
     "ising_batch_cluster_size": (ctypes.c_int, [_vp, _P(_i32)]),
+    "ising_batch_last_run": (ctypes.c_int, [_vp, _P(_i32), _P(_i64)]),
+    "ising_last_run": (ctypes.c_int, [_vp, _P(_i32), _P(_i64)]),
     "ising_batch_observables_ex": (ctypes.c_int, [_vp, _i32, _P(_i64), _P(_i64), _P(_i64)]),
     "ising_batch_history": (ctypes.c_int, [_vp, _i32, _i64, _i64, _P(_i64), _P(_i64)]),
     "ising_batch_moments": (ctypes.c_int, [_vp, _i32, _i64, _P(_d), _P(_u64)]),
@@ -221,12 +223,20 @@ def ising_batch_observables(b: int, idx: int) -> tuple[int, int]:
 
 SPECIALIZE_OFF, SPECIALIZE_AUTO, SPECIALIZE_ALWAYS = 0, 1, 2
 CLUSTER_OFF, CLUSTER_AUTO, CLUSTER_ALWAYS = 0, 1, 2
+RUN_NONE, RUN_TILED, RUN_AHEAD, RUN_CLUSTER, RUN_BYTES, RUN_CUBIC = range(6)
 
 
 def ising_set_specialize(mode: int) -> None:
     """Process-wide: whether handles created afterwards sweep with a kernel compiled
     for their thresholds (SPECIALIZE_OFF, _AUTO (default), _ALWAYS)."""
     _check(lib().ising_set_specialize(int(mode)))
+
+
+def ising_last_run(h: int) -> tuple[int, int]:
+    """(form RUN_*, kernels enqueued) of the handle's last run."""
+    form, launches = ctypes.c_int32(), ctypes.c_int64()
+    _check(lib().ising_last_run(h, ctypes.byref(form), ctypes.byref(launches)))
+    return form.value, launches.value
 
 
 def ising_specialized(h: int) -> tuple[bool, str]:
@@ -399,6 +409,10 @@ class Lattice:
     def synchronize(self) -> None:
         ising_synchronize(self.h)
 
+    def last_run(self) -> tuple[int, int]:
+        """(RUN_* form, kernels enqueued) of the last run."""
+        return ising_last_run(self.h)
+
     def specialized(self) -> tuple[bool, str]:
         """(True, note) when the sweeps run a kernel compiled for this lattice's thresholds."""
         return ising_specialized(self.h)
@@ -487,6 +501,12 @@ class Batch:
         out = np.empty((L, L), dtype=np.int8)
         _check(lib().ising_batch_get_lattice(self.b, int(idx), _ptr(out, ctypes.c_int8)))
         return out
+
+    def last_run(self) -> tuple[int, int]:
+        """(RUN_* form, kernels enqueued) of the last run."""
+        form, launches = ctypes.c_int32(), ctypes.c_int64()
+        _check(lib().ising_batch_last_run(self.b, ctypes.byref(form), ctypes.byref(launches)))
+        return form.value, launches.value
 
     def specialized(self) -> bool:
         """True while the batch sweeps with a kernel compiled for its one temperature."""
