@@ -101,8 +101,8 @@ int ising_init(ising_t *out, int64_t L, double beta, uint64_t seed);
  * until ising_free); NULL makes the handle create and own a non-blocking stream.  Device memory: packed L*L/8
  * bytes, int8 L*L bytes, plus 16 bytes of history per sweep (grown on demand); packed
  * sides up to 8192 take a workspace for random numbers drawn ahead as well (2 to 16 MB up
- * to L = 192, at most 16 L^2 bytes beyond, taken by the first run that reaches 16 sweeps; where
- * it cannot be had, the sweeps run without it).
+ * to L = 192, at most 16 L^2 bytes beyond, taken by the first run that reaches 16 sweeps in all --
+ * 96 at L = 64, 64 at 128, 32 at 192; where it cannot be had, the sweeps run without it).
  * Errors: EINVAL (L, beta, start, kernel), ENOMEM, ECUDA.
  */
 int ising_init_ex(ising_t *out, int64_t L, double beta, uint64_t seed, int start, int kernel, void *stream);
@@ -271,6 +271,7 @@ int ising_batch_cluster_size(ising_batch_t b, int32_t *cluster_size);
 #define ISING_RUN_CLUSTER 3  /* batches: lattices resident in thread-block clusters */
 #define ISING_RUN_BYTES 4    /* the int8 kernel */
 #define ISING_RUN_CUBIC 5    /* three dimensions, one launch per half-sweep */
+#define ISING_RUN_RESIDENT 6 /* L <= 256: one launch, the lattice in one CTA's shared memory */
 int ising_last_run(ising_t h, int32_t *form, int64_t *launches);
 int ising_batch_last_run(ising_batch_t b, int32_t *form, int64_t *launches);
 

@@ -638,18 +638,21 @@ int setup_ahead(ising_t h)
     return ISING_OK;
 }
 
-// Whether a run of n sweeps goes that way.  The workspace (two mask buffers, for lattices of
+// Whether a run of n sweeps can go that way.  The workspace (two mask buffers, for lattices of
 // several tiles two copies of the planes, the drawing tickets) is allocated by the first run
-// that needs it once the handle has been asked for 16 sweeps in all: it costs about 0.1 ms, the
-// tiled kernel's time for 10 sweeps of a lattice this size.  Before that, where memory is short
-// and on a stream that is being captured, the tiled kernel runs; the chain is the same.
-constexpr int64_t kAheadMinSweeps = 16;
+// that needs it once the handle has been asked for 16 sweeps in all, of lattices that the resident
+// kernel sweeps for 96 (L = 64), 64 (128) and 32 (192): it costs about 70 us, the other kernel's
+// time for that many (us for all sweeps of a new handle, allocating / not: L = 64, 96 sweeps
+// 110 / 113; 128, 64 104 / 105; 192, 32 110 / 114).  Before that, where memory is short and on a stream
+// that is being captured, the resident or the tiled kernel runs; the chain is the same.
+int64_t ahead_min_sweeps(int64_t L) { return L <= 192 ? 128 - L / 2 : 16; }
 bool ahead_ready(ising_t h, int64_t n)
 {
     const AheadPlan& p = h->ahead_plan;
     if (p.tiles == 0) return false;
-    if (h->ahead_ws || ahead_alone(h->ahead, n)) return true;
-    if (h->ahead_refused || h->sweeps_done + n < kAheadMinSweeps) return false;
+    if (h->ahead_ws) return true;
+    const int64_t least = h->kernel == kKernelCubic ? 16 : ahead_min_sweeps(h->L);
+    if (h->ahead_refused || h->sweeps_done + n < least) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
@@ -670,6 +673,25 @@ bool ahead_ready(ising_t h, int64_t n)
     a.masks[1] = reinterpret_cast<uint2*>(ws + 256 + p.mask_bytes);
     a.copy = reinterpret_cast<uint32_t*>(ws + 256 + 2 * p.mask_bytes);
     return true;
+}
+
+// The form of a run of n sweeps.  Up to L = 256 the resident kernel takes the runs that are over before a
+// launch to draw and one to update would be, and whatever cannot be drawn ahead; of L = 64, runs of
+// 4 to 8 sweeps draw their own masks in one launch.  us from the call to its end, resident / drawn
+// ahead: L = 64, 3 sweeps 14.3 / 13.8, 4 15.1 / 14.1, 8 19.8 / 15.3; L = 128, 1 12.7 / 14.2, 5 18.2 / 18.7,
+// 6 20.0 / 19.1; L = 192, 2 18.1 / 18.9, 3 21.2 / 19.6; L = 256, 1 16.2 / 19.7, 2 20.4 / 19.5.  (Two
+// launches of the tiled kernel a sweep: 15 sweeps of a new handle of L = 64 106, resident 29;
+// L = 256 159 and 82.)
+int run_form(ising_t h, int64_t n)
+{
+    const int other = h->kernel == kKernelCubic ? ISING_RUN_CUBIC : h->kernel == ISING_INT8 ? ISING_RUN_BYTES : ISING_RUN_TILED;
+    if (h->ahead_plan.tiles == 0) return other;
+    if (other == ISING_RUN_TILED && h->L <= packed_resident_max_L()) {
+        if (n >= 4 && ahead_alone(h->ahead, n)) return ISING_RUN_AHEAD;
+        if (n * std::max<int64_t>(h->L * h->L, 16384) <= 81920 || !ahead_ready(h, n)) return ISING_RUN_RESIDENT;
+        return ISING_RUN_AHEAD;
+    }
+    return ahead_ready(h, n) ? ISING_RUN_AHEAD : other;
 }
 
 int check_handle(ising_t h)
@@ -936,11 +958,11 @@ int ising_init_ex(ising_t* out, int64_t L, double beta, uint64_t seed, int start
         d.sweep = 0;
         d.target = kNoTarget;
         d.active = 1;
-        // the sweep kernel: the resident one for small sides, else the tiled one, compiled
-        // for this lattice's thresholds where the mode asks for it and it can be had
+        // the tiled kernel, compiled for this lattice's thresholds where the mode asks for it and it
+        // can be had (run_form: what small sides sweep with)
         const void* fixed = nullptr;
         const int mode = g_specialize.load();
-        if (L <= 256) {
+        if (L <= packed_resident_max_L()) {
             h->kernel_note = "built-in: L <= 256";
         } else if (mode == ISING_SPECIALIZE_OFF) {
             h->kernel_note = "built-in: specialisation switched off";
@@ -1096,17 +1118,25 @@ int ising_sweep(ising_t h, int64_t n)
     if (n == 0) return ISING_OK;
     rc = ensure_hist(h, h->sweeps_done + n);
     if (rc) return rc;
-    if (ahead_ready(h, n)) {
+    const int form = run_form(h, n);
+    int64_t launched = 0;
+    if (form == ISING_RUN_AHEAD) {
         h->ahead.hist = h->hist;
-        int64_t launched = 0;
         CK(launch_ahead_sweeps(h->ahead, h->ahead_plan.chunk, (uint32_t)h->sweeps_done, n, h->stream, &launched));
-        h->last = {ISING_RUN_AHEAD, launched};
-    } else if (h->kernel == ISING_PACKED) {
+    } else if (form == ISING_RUN_RESIDENT) {
+        LatticeDesc d = h->desc;
+        for (int64_t done = 0; done < n; ++launched) {
+            const int64_t chunk = std::min<int64_t>(n - done, 4096);
+            d.sweep = (uint32_t)(h->sweeps_done + done);
+            CK(launch_packed_resident(d, (int)chunk, h->stream));
+            done += chunk;
+        }
+    } else if (form == ISING_RUN_TILED) {
         rc = h->eng.run(n, 0);
         if (rc) return rc;
-        h->last = {ISING_RUN_TILED, h->eng.launched};
-    } else if (h->kernel == kKernelCubic) {
-        h->last = {ISING_RUN_CUBIC, 2 * n};
+        launched = h->eng.launched;
+    } else if (form == ISING_RUN_CUBIC) {
+        launched = 2 * n;
         const CubicDesc d = cubic_desc(h);
         for (int64_t k = 0; k < n; ++k)
             for (int c = 0; c < 2; ++c) {
@@ -1115,7 +1145,7 @@ int ising_sweep(ising_t h, int64_t n)
                 if (e != cudaSuccess) return cuda_fail(e, "3D half-sweep launch");
             }
     } else {
-        h->last = {ISING_RUN_BYTES, 2 * n};
+        launched = 2 * n;
         uint32_t t2, t4, all2, all4;
         LatticeDesc tmp{};
         set_thresholds(tmp, h->T);
@@ -1132,6 +1162,7 @@ int ising_sweep(ising_t h, int64_t n)
             }
         }
     }
+    h->last = {form, launched};
     h->sweeps_done += n;
     h->desc.sweep = (uint32_t)h->sweeps_done;
     return ISING_OK;

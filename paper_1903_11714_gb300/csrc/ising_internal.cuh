@@ -128,6 +128,10 @@ bool ahead_alone(const AheadLattice& d, int64_t n);
 // Enqueues n sweeps, numbered from `sweep` on, in launches of at most `chunk` sweeps, added to *launched.
 cudaError_t launch_ahead_sweeps(const AheadLattice& d, int chunk, uint32_t sweep, int64_t n, cudaStream_t s,
                                 int64_t* launched);
+// One small lattice (L <= packed_resident_max_L()) swept nsweeps times by a single
+// CTA holding both planes in shared memory; writes hist[d.sweep .. +nsweeps).
+int packed_resident_max_L();
+cudaError_t launch_packed_resident(const LatticeDesc& d, int nsweeps, cudaStream_t s);
 cudaError_t launch_packed_advance(LatticeDesc* desc, const int32_t* count, int max_count, int steps,
                                   cudaStream_t s);
 // Cluster-resident sweeps (sweep_cluster.cu): lattices of one side L <= cluster_max_L()

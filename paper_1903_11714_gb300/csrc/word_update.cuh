@@ -1,6 +1,7 @@
 // The Metropolis update of 32-site words of a target colour plane (paper Sec. 3.1
 // acceptance rule on the bit-packed colour planes of Sec. 3.2), shared by the
-// tiled sweep kernel, the int8 kernel and the three-dimensional sweep.
+// tiled sweep kernel, the single-CTA resident kernel, the int8 kernel and the
+// three-dimensional sweep.
 #pragma once
 #include "ising_device.cuh"
 

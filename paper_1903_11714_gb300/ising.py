@@ -223,7 +223,7 @@ def ising_batch_observables(b: int, idx: int) -> tuple[int, int]:
 
 SPECIALIZE_OFF, SPECIALIZE_AUTO, SPECIALIZE_ALWAYS = 0, 1, 2
 CLUSTER_OFF, CLUSTER_AUTO, CLUSTER_ALWAYS = 0, 1, 2
-RUN_NONE, RUN_TILED, RUN_AHEAD, RUN_CLUSTER, RUN_BYTES, RUN_CUBIC = range(6)
+RUN_NONE, RUN_TILED, RUN_AHEAD, RUN_CLUSTER, RUN_BYTES, RUN_CUBIC, RUN_RESIDENT = range(7)
 
 
 def ising_set_specialize(mode: int) -> None:

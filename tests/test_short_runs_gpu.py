@@ -1,0 +1,62 @@
+"""Runs of small lattices that are too short, or too early, for random numbers drawn ahead: one launch
+of the resident kernel (L <= 256), before and after longer runs, and captured into a graph."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1903_11714_gb300 import build as libbuild
+from paper_1903_11714_gb300 import ising
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    libbuild.build()
+    ising.lib()
+
+
+RESIDENT, AHEAD = (ising.RUN_RESIDENT, 1), ising.RUN_AHEAD
+
+
+def check(lat, L, beta, seed, n):
+    ref, M, E, _ = oracle.run(L, beta, seed, ising.HOT, n)
+    m, e = lat.history(0, n)
+    assert np.array_equal(m, M) and np.array_equal(e, E)
+    assert np.array_equal(lat.get_lattice(), ref)
+
+
+# (run, form): a new handle's first runs, one long enough to take the workspace, then the lengths on
+# either side of where a launch to draw and one to update are the faster
+@pytest.mark.parametrize("L,runs", [
+    (64, [(1, RESIDENT), (15, RESIDENT), (70, RESIDENT), (30, AHEAD), (1, RESIDENT), (3, RESIDENT), (4, AHEAD), (8, AHEAD), (9, AHEAD)]),
+    (128, [(1, RESIDENT), (15, RESIDENT), (47, RESIDENT), (20, AHEAD), (1, RESIDENT), (5, RESIDENT), (6, AHEAD)]),
+    (192, [(1, RESIDENT), (15, RESIDENT), (40, AHEAD), (2, RESIDENT), (3, AHEAD)]),
+    (256, [(1, RESIDENT), (14, RESIDENT), (17, AHEAD), (1, RESIDENT), (2, AHEAD)]),
+])
+@pytest.mark.parametrize("beta", [0.0, 0.4406868, 200.0])
+def test_forms_and_chain(L, runs, beta):
+    lat = ising.Lattice(L, beta, 11 + L, ising.HOT)
+    for n, form in runs:
+        lat.sweep(n)
+        assert lat.last_run() == form if form == RESIDENT else lat.last_run()[0] == form
+    check(lat, L, beta, 11 + L, sum(n for n, _ in runs))
+    lat.close()
+
+
+@pytest.mark.parametrize("L", [64, 128, 192, 256])
+def test_captured_at_once(L):
+    # a program that captures its run right after it made the handle
+    import torch
+
+    stream = torch.cuda.Stream()
+    lat = ising.Lattice(L, 0.43, 32, ising.HOT, stream=stream)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+        lat.sweep(100)
+    assert lat.last_run() == RESIDENT
+    with torch.cuda.stream(stream):
+        g.replay()
+    check(lat, L, 0.43, 32, 100)
+    del g
+    lat.close()
