@@ -691,6 +691,11 @@ int run_form(ising_t h, int64_t n)
         if (n * std::max<int64_t>(h->L * h->L, 16384) <= 81920 || !ahead_ready(h, n)) return ISING_RUN_RESIDENT;
         return ISING_RUN_AHEAD;
     }
+    // One or two sweeps of a large lattice: the launch that draws has nothing to update and the one that
+    // updates nothing to draw, and the planes are copied once.  us from the call to its end, tiled /
+    // drawn ahead: one sweep of L = 5,120 33.9 / 33.1, 5,504 35.0 / 35.0, 6,144 35.1 / 41.1, 8,192 40.3 / 51.6; two of
+    // 6,144 58.0 / 55.6, 7,168 67.7 / 63.8, 8,192 68.2 / 74.0; three of 8,192 96.0 / 95.9.
+    if (other == ISING_RUN_TILED && (n == 1 ? h->L > 5504 : n == 2 && h->L > 7168)) return other;
     return ahead_ready(h, n) ? ISING_RUN_AHEAD : other;
 }
 

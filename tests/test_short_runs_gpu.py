@@ -1,5 +1,6 @@
-"""Runs of small lattices that are too short, or too early, for random numbers drawn ahead: one launch
-of the resident kernel (L <= 256), before and after longer runs, and captured into a graph."""
+"""Runs that are too short, or too early, for random numbers drawn ahead: one launch of the resident
+kernel (L <= 256) or two a sweep of the tiled one (large lattices), before and after longer runs, and
+captured into a graph."""
 import numpy as np
 import pytest
 
@@ -60,3 +61,22 @@ def test_captured_at_once(L):
     check(lat, L, 0.43, 32, 100)
     del g
     lat.close()
+
+
+@pytest.mark.parametrize("L,runs", [(5504, [(20, AHEAD), (1, AHEAD), (2, AHEAD)]),
+                                    (5568, [(20, AHEAD), (1, ising.RUN_TILED), (2, AHEAD)]),
+                                    (8192, [(20, AHEAD), (1, ising.RUN_TILED), (2, ising.RUN_TILED), (3, AHEAD)])])
+def test_one_or_two_sweeps_of_large_lattices(L, runs):
+    lat = ising.Lattice(L, 0.43, 6, ising.HOT)
+    n = sum(r for r, _ in runs)
+    for r, form in runs:
+        lat.sweep(r)
+        assert lat.last_run()[0] == form
+    b = ising.Batch(1, L, L * L // 8 + 16 * n + 4096)
+    b.set_cluster(ising.CLUSTER_OFF)
+    k = b.add(L, 0.43, 6, ising.HOT, n)
+    b.run(n)
+    assert all(np.array_equal(x, y) for x, y in zip(lat.history(0, n), b.history(k)))
+    assert np.array_equal(lat.get_lattice(), b.get_lattice(k))
+    lat.close()
+    b.close()
