@@ -245,7 +245,7 @@ int ising_batch_specialized(ising_batch_t b, int32_t *specialized);
  * In the automatic mode a batch of sides up to 4,096 (whole-row tiles, several
  * temperatures) and up to about 1e8 sites is swept with its random numbers drawn ahead
  * of the update instead where that is estimated to be faster (any mix of sides; most
- * batches of up to 5e7 sites): from its 16th sweep on, in a device workspace beside the
+ * batches of up to 5e7 sites): from its 32nd sweep on, in a device workspace beside the
  * arena of about 4 bytes a site, taken by the first such run; where it cannot be had,
  * the other two forms run.  The chain is the same, bit for bit.
  * Paper: Sec. 3.1 (the schedule), Sec. 4.1 (scans of small lattices).

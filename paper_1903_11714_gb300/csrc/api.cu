@@ -550,7 +550,7 @@ struct ising_batch_s {
     // launches), and whether its tables follow the slots
     bool ahead_wanted = false, ahead_refused = false, ahead_tables = false;
     AheadBatch ahead{};
-    int64_t ahead_steps = 0, ahead_asked = 0;
+    int64_t ahead_steps = 0, ahead_asked = 0, ahead_sites = 0;
     char* ahead_ws = nullptr;
     int64_t ahead_ws_bytes = 0;
     std::vector<void*> ahead_outgrown;
@@ -1575,6 +1575,7 @@ void update_ahead(ising_batch_t b)
     }
     if (drawn_ahead >= other) return;
     b->ahead_wanted = true;
+    b->ahead_sites = sites;
     b->ahead.chunk = ahead_batch_chunk(longest);
     // tall tiles once a launch has work for every SM (us a sweep, low / tall tiles: 8 x 256
     // 0.75 / 1.08; 32 x 256 1.53 / 1.23; 16 x 512 2.40 / 2.36; 64 x 1,024 32.2 / 29.0)
@@ -1582,16 +1583,33 @@ void update_ahead(ising_batch_t b)
 }
 
 // Whether a run of n sweeps goes that way: the workspace and the tables are made ready by the
-// first run that needs them, once the batch has been asked for 16 sweeps in all.  Before that,
+// first run that needs them, once the batch has been asked for 32 sweeps in all (us for the first
+// run of a new batch, with the workspace's allocation / without: 16 sweeps of 8 x 1,024 180 / 159, of
+// 48 x 1,024 496 / 422; 32 sweeps 232 / 300 and 813 / 821).  Before that,
 // where memory is short and on a stream that is being captured: the tiled or the
 // cluster-resident kernel, as otherwise (the launches here carry the batch's tables by value, so
 // a graph of them would not follow a batch that changes between its replays).
-constexpr int64_t kAheadMinBatchSweeps = 16;
+//
+// Runs of up to four sweeps have a launch that draws with nothing to update and one that updates
+// with nothing to draw: one sweep is left to the other forms, two from 5e6 sites on, three from 3e7
+// and four from 8e7.  us from the call to its end, others / drawn ahead: one sweep of 16 x 64 20.2 / 23.5,
+// 8 x 256 23.5 / 24.4, 8 x 2,048 29.9 / 48.5; two of 32 x 256 31.8 / 26.1, 16 x 512 32.7 / 31.1, 8 x 1,024
+// 34.7 / 33.8, 20 lattices of up to 1,024 (5.6e6 sites, a graph) 28.6 / 32.1, 8 x 2,048 49.4 / 62.8; three of
+// 4,096 + 2,048 + 1,024 (2.2e7 sites) 62.9 / 62.9, 8 x 2,048 68.5 / 75.3, 20 x 2,048 148 / 164; four of 8 x 2,048
+// 89.2 / 88.7, 20 x 2,048 194 / 199.
+bool ahead_run_too_short(int64_t sites, int64_t n)
+{
+    constexpr int64_t kFrom[] = {0, 0, 5000000, 30000000, 80000000};
+    return n <= 4 && sites >= kFrom[n];
+}
+
+constexpr int64_t kAheadMinBatchSweeps = 32;
 int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
 {
     *ready = false;
     b->ahead_asked = std::min<int64_t>(b->ahead_asked + n, kAheadMinBatchSweeps);
-    if (!b->ahead_wanted || b->ahead_refused || b->ahead_asked < kAheadMinBatchSweeps) return ISING_OK;
+    if (!b->ahead_wanted || b->ahead_refused || b->ahead_asked < kAheadMinBatchSweeps || ahead_run_too_short(b->ahead_sites, n))
+        return ISING_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
         cudaGetLastError();

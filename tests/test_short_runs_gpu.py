@@ -80,3 +80,21 @@ def test_one_or_two_sweeps_of_large_lattices(L, runs):
     assert np.array_equal(lat.get_lattice(), b.get_lattice(k))
     lat.close()
     b.close()
+
+
+# batches: one sweep, two from 5e6 sites on, three from 3e7 and four from 8e7 on go to the kernels that draw as they go
+@pytest.mark.parametrize("Ls,shortest", [([64, 320, 512], 2), ([2048, 1024, 512, 64], 3), ([4096, 4096], 4), ([4096] * 5, 5)])
+@pytest.mark.parametrize("graph", [False, True])
+def test_short_batch_runs(Ls, shortest, graph):
+    runs, out = [35, 1, 2, 3, 4, 5], []
+    for mode in (ising.CLUSTER_AUTO, ising.CLUSTER_OFF):
+        b = ising.Batch(len(Ls), max(Ls), sum(L * L // 8 + 16 * 50 + 4096 for L in Ls) + (1 << 25))
+        b.set_cluster(mode)
+        idx = [b.add(L, 0.35 + 0.05 * k, 70 + k, ising.HOT, 50) for k, L in enumerate(Ls)]
+        for n in runs:
+            b.run(n, n if graph else 0)
+            assert (b.last_run()[0] == ising.RUN_AHEAD) == (mode == ising.CLUSTER_AUTO and n >= shortest)
+        out.append([(*b.history(i), b.get_lattice(i)) for i in idx])
+        b.close()
+    for short, tiled in zip(*out):
+        assert all(np.array_equal(a, t) for a, t in zip(short, tiled))
