@@ -102,7 +102,7 @@ int ising_init(ising_t *out, int64_t L, double beta, uint64_t seed);
  * bytes, int8 L*L bytes, plus 16 bytes of history per sweep (grown on demand); packed
  * sides up to 8192 take a workspace for random numbers drawn ahead as well (2 to 16 MB up
  * to L = 192, at most 16 L^2 bytes beyond, taken by the first run that reaches 16 sweeps in all --
- * 96 at L = 64, 64 at 128, 32 at 192; where it cannot be had, the sweeps run without it).
+ * 96 at L = 64, 64 at 128, 32 at 192; see ising_set_workspace).
  * Errors: EINVAL (L, beta, start, kernel), ENOMEM, ECUDA.
  */
 int ising_init_ex(ising_t *out, int64_t L, double beta, uint64_t seed, int start, int kernel, void *stream);
@@ -258,6 +258,20 @@ int ising_batch_set_cluster(ising_batch_t b, int32_t mode);
 int ising_batch_cluster_size(ising_batch_t b, int32_t *cluster_size);
 
 /*
+ * The workspace for random numbers drawn ahead (ising_init_ex, ising_init3d: sides 64 and
+ * 128).  mode ISING_WORKSPACE_BESIDE (the default): taken by the first run that gains by it,
+ * kept until the handle is freed.  All workspaces of the process together hold at most 4 GB, and
+ * one of more than 4 MB takes at most a 64th of the device memory then free; where it cannot be had, the sweeps
+ * run without it and it is tried again after 1,024 more.  ISING_WORKSPACE_NONE: never, and one held is
+ * given back at once (the call then synchronises; a graph captured from a run that used
+ * it must not be replayed any more).  The chain is the same either way, bit for bit.
+ * Paper: none (memory of the Sec. 3.1 sweep).  Errors: EINVAL (null handle, mode), ECUDA.
+ */
+#define ISING_WORKSPACE_NONE 0
+#define ISING_WORKSPACE_BESIDE 1
+int ising_set_workspace(ising_t h, int32_t mode);
+
+/*
  * What the last run with n > 0 sweeps was (ising_sweep; ising_batch_run): *form, the kernels
  * it took, and *launches, how many it enqueued (those inside replayed graphs counted
  * one by one).  The forms give the same chain bit for bit; which one runs follows from the
@@ -299,7 +313,8 @@ int ising_thresholds3d(double beta, uint64_t T[3]);
 
 /*
  * Creates a bit-packed cubic lattice of side L (L % 64 == 0, 64 <= L <= 8192):
- * device memory L^3/8 bytes of planes plus 16 bytes of history per sweep.
+ * device memory L^3/8 bytes of planes plus 16 bytes of history per sweep, and for sides 64 and
+ * 128 a workspace of 17 and 4 MB (ising_set_workspace).
  * start and stream as in ising_init_ex.  The handle works with ising_sweep,
  * ising_observables, ising_history, ising_moments[_ex] (N = L^3), ising_get_lattice
  * (out[L^3], index (i*L + j)*L + k), ising_get_planes / ising_set_planes (L*L

@@ -491,6 +491,64 @@ struct LastRun {
     }
 };
 
+// Relaxes this thread's stream capture mode: a workspace may be needed for the first time while
+// another thread captures a graph on a stream of its own, which forbids allocations in its
+// strictest mode unless this thread relaxes its own.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Device memory that makes sweeps faster and that they can do without.  So that it never stands in
+// the way of what a program allocates itself, all workspaces of the process together hold at
+// most kTotal, and one beyond kSmall takes at most a 64th of the device memory that is free when it
+// is taken (the question takes 15 us, half of what a new handle of L = 320 takes for 16 sweeps).
+struct Workspace {
+    static constexpr int64_t kTotal = 4ll << 30, kSmall = 4ll << 20;
+    static std::atomic<int64_t> held;
+    char* p = nullptr;
+    int64_t bytes = 0;
+
+    // The most that take() would give now.
+    static int64_t room()
+    {
+        RelaxedCapture relaxed;
+        size_t free = 0, total = 0;
+        if (cudaMemGetInfo(&free, &total) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        return std::max<int64_t>(0, std::min<int64_t>(kTotal - held.load(), (int64_t)(free / 64)));
+    }
+    bool take(int64_t n)
+    {
+        if (n > kSmall && n > room()) return false;
+        if (held.fetch_add(n) + n <= kTotal) {
+            RelaxedCapture relaxed;
+            if (cudaMalloc(&p, (size_t)n) == cudaSuccess) {
+                bytes = n;
+                return true;
+            }
+            cudaGetLastError();
+            p = nullptr;
+        }
+        held.fetch_sub(n);
+        return false;
+    }
+    // (the caller has waited for the work that uses it)
+    void give()
+    {
+        if (!p) return;
+        RelaxedCapture relaxed;
+        cudaFree(p);
+        held.fetch_sub(bytes);
+        p = nullptr;
+        bytes = 0;
+    }
+};
+std::atomic<int64_t> Workspace::held{0};
+
 // A handle's or batch's share in the report blocks (report_block.h).
 struct ReadbackUser {
     ReadbackUser() { readback_user(1); }
@@ -524,8 +582,9 @@ struct ising_s {
     std::string kernel_note;    // which sweep kernel runs, and why (ising_specialized)
     AheadLattice ahead{};       // packed, built-in kernel, L <= ahead_max_L(): the sweep with its
     AheadPlan ahead_plan;       // random numbers drawn ahead (tiles = 0: the tiled kernel)
-    void* ahead_ws = nullptr;
-    bool ahead_refused = false; // no memory for the workspace
+    Workspace ahead_ws;
+    int64_t ahead_from = 0;     // sweeps in all from which a run may take the workspace
+    bool ahead_declined = false;  // ising_set_workspace
     const void* cubic_fixed[2] = {nullptr, nullptr};  // 3D: the colours' compiled instances
 };
 
@@ -595,17 +654,17 @@ int ensure_hist(ising_t h, int64_t need)
 uint32_t thr32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : (uint32_t)T; }
 uint32_t all32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : 0u; }
 
-// cudaMalloc for a workspace that a sweep call may need for the first time while another thread
-// captures a graph on a stream of its own: such a capture forbids the call in its strictest mode
-// unless this thread relaxes its own.
 cudaError_t malloc_relaxed(char** p, size_t bytes)
 {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    const cudaError_t e = cudaMalloc(p, bytes);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    return e;
+    RelaxedCapture relaxed;
+    return cudaMalloc(p, bytes);
 }
+
+// Sweeps in all from which a run takes the workspace: 16; of lattices that the resident kernel
+// sweeps, 96 (L = 64), 64 (128) and 32 (192).  It costs about 70 us, the other kernel's time for that
+// many (us for all sweeps of a new handle, allocating / not: L = 64, 96 sweeps 110 / 113; 128, 64 104 /
+// 105; 192, 32 110 / 114).
+int64_t ahead_min_sweeps(int64_t L) { return L <= 192 ? 128 - L / 2 : 16; }
 
 // The sweep with its random numbers drawn ahead: the lattice's plan and constants.
 int setup_ahead(ising_t h)
@@ -615,6 +674,7 @@ int setup_ahead(ising_t h)
     if (p.tiles == 0) return ISING_OK;
     CK(ahead_configure(p));
     h->ahead_plan = p;
+    h->ahead_from = cube ? 16 : ahead_min_sweeps(h->L);
     AheadLattice& a = h->ahead;
     a.home = h->planes;
     a.status = h->eng.d_status;
@@ -640,33 +700,32 @@ int setup_ahead(ising_t h)
 
 // Whether a run of n sweeps can go that way.  The workspace (two mask buffers, for lattices of
 // several tiles two copies of the planes, the drawing tickets) is allocated by the first run
-// that needs it once the handle has been asked for 16 sweeps in all, of lattices that the resident
-// kernel sweeps for 96 (L = 64), 64 (128) and 32 (192): it costs about 70 us, the other kernel's
-// time for that many (us for all sweeps of a new handle, allocating / not: L = 64, 96 sweeps
-// 110 / 113; 128, 64 104 / 105; 192, 32 110 / 114).  Before that, where memory is short and on a stream
-// that is being captured, the resident or the tiled kernel runs; the chain is the same.
-int64_t ahead_min_sweeps(int64_t L) { return L <= 192 ? 128 - L / 2 : 16; }
+// that needs it once the handle has been asked for ahead_min_sweeps in all.  Before that, where
+// it cannot be had (tried again after kAheadRetry more sweeps) and on a stream that is being
+// captured, the resident or the tiled kernel runs; the chain is the same.
+constexpr int64_t kAheadRetry = 1024;
 bool ahead_ready(ising_t h, int64_t n)
 {
     const AheadPlan& p = h->ahead_plan;
-    if (p.tiles == 0) return false;
-    if (h->ahead_ws) return true;
-    const int64_t least = h->kernel == kKernelCubic ? 16 : ahead_min_sweeps(h->L);
-    if (h->ahead_refused || h->sweeps_done + n < least) return false;
+    if (p.tiles == 0 || h->ahead_declined) return false;
+    if (h->ahead_ws.p) return true;
+    if (h->sweeps_done + n < h->ahead_from) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
         return false;
     }
-    char* ws = nullptr;
-    if (malloc_relaxed(&ws, (size_t)(2 * p.mask_bytes + p.copy_bytes + 256)) != cudaSuccess ||
-        cudaMemsetAsync(ws, 0, 256, h->stream) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(ws);
-        h->ahead_refused = true;
+    if (!h->ahead_ws.take(2 * p.mask_bytes + p.copy_bytes + 256)) {
+        h->ahead_from = h->sweeps_done + n + kAheadRetry;
         return false;
     }
-    h->ahead_ws = ws;
+    char* ws = h->ahead_ws.p;
+    if (cudaMemsetAsync(ws, 0, 256, h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        h->ahead_ws.give();
+        h->ahead_from = h->sweeps_done + n + kAheadRetry;
+        return false;
+    }
     AheadLattice& a = h->ahead;
     a.ticket = reinterpret_cast<int*>(ws);
     a.masks[0] = reinterpret_cast<uint2*>(ws + 256);
@@ -878,7 +937,7 @@ void destroy_handle(ising_t h)
     cudaFree(h->hist);
     cudaFree(h->d_me0);
     cudaFree(h->d_work3);
-    cudaFree(h->ahead_ws);
+    h->ahead_ws.give();
     cudaFree(h->d_read);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
     delete h;
@@ -1170,6 +1229,20 @@ int ising_sweep(ising_t h, int64_t n)
     h->last = {form, launched};
     h->sweeps_done += n;
     h->desc.sweep = (uint32_t)h->sweeps_done;
+    return ISING_OK;
+}
+
+int ising_set_workspace(ising_t h, int32_t mode)
+{
+    const int rc = check_handle(h);
+    if (rc) return rc;
+    if (mode != ISING_WORKSPACE_NONE && mode != ISING_WORKSPACE_BESIDE)
+        return fail(ISING_EINVAL, "workspace mode %d is not 0 or 1", mode);
+    h->ahead_declined = mode == ISING_WORKSPACE_NONE;
+    if (h->ahead_declined && h->ahead_ws.p) {
+        CK(cudaStreamSynchronize(h->stream));
+        h->ahead_ws.give();
+    }
     return ISING_OK;
 }
 

@@ -69,6 +69,7 @@ _SIGS = {
     "ising_batch_set_cluster": (ctypes.c_int, [_vp, _i32]),
     "ising_batch_cluster_size": (ctypes.c_int, [_vp, _P(_i32)]),
     "ising_batch_last_run": (ctypes.c_int, [_vp, _P(_i32), _P(_i64)]),
+    "ising_set_workspace": (ctypes.c_int, [_vp, _i32]),
     "ising_last_run": (ctypes.c_int, [_vp, _P(_i32), _P(_i64)]),
     "ising_batch_observables_ex": (ctypes.c_int, [_vp, _i32, _P(_i64), _P(_i64), _P(_i64)]),
     "ising_batch_history": (ctypes.c_int, [_vp, _i32, _i64, _i64, _P(_i64), _P(_i64)]),
@@ -223,6 +224,7 @@ def ising_batch_observables(b: int, idx: int) -> tuple[int, int]:
 
 SPECIALIZE_OFF, SPECIALIZE_AUTO, SPECIALIZE_ALWAYS = 0, 1, 2
 CLUSTER_OFF, CLUSTER_AUTO, CLUSTER_ALWAYS = 0, 1, 2
+WORKSPACE_NONE, WORKSPACE_BESIDE = 0, 1
 RUN_NONE, RUN_TILED, RUN_AHEAD, RUN_CLUSTER, RUN_BYTES, RUN_CUBIC, RUN_RESIDENT = range(7)
 
 
@@ -230,6 +232,12 @@ def ising_set_specialize(mode: int) -> None:
     """Process-wide: whether handles created afterwards sweep with a kernel compiled
     for their thresholds (SPECIALIZE_OFF, _AUTO (default), _ALWAYS)."""
     _check(lib().ising_set_specialize(int(mode)))
+
+
+def ising_set_workspace(h: int, mode: int) -> None:
+    """WORKSPACE_BESIDE (default) or WORKSPACE_NONE: whether the handle may take device memory to
+    draw random numbers ahead (given back at once by WORKSPACE_NONE)."""
+    _check(lib().ising_set_workspace(h, int(mode)))
 
 
 def ising_last_run(h: int) -> tuple[int, int]:
@@ -408,6 +416,9 @@ class Lattice:
 
     def synchronize(self) -> None:
         ising_synchronize(self.h)
+
+    def set_workspace(self, mode: int) -> None:
+        ising_set_workspace(self.h, mode)
 
     def last_run(self) -> tuple[int, int]:
         """(RUN_* form, kernels enqueued) of the last run."""
