@@ -245,8 +245,9 @@ int ising_batch_specialized(ising_batch_t b, int32_t *specialized);
  * In the automatic mode a batch of sides up to 4,096 (whole-row tiles, several
  * temperatures) and up to about 1e8 sites is swept with its random numbers drawn ahead
  * of the update instead where that is estimated to be faster (any mix of sides; most
- * batches of up to 5e7 sites): from its 32nd sweep on, in a device workspace beside the
- * arena of about 4 bytes a site, taken by the first such run; where it cannot be had,
+ * batches of up to 5e7 sites): from its 32nd sweep on, in a device workspace of 8.25
+ * bytes a site for sides up to 2,048 (longer sides 4.25), at most 1.1 GB, beside the arena
+ * (ising_batch_set_workspace), taken by the first such run; where it cannot be had,
  * the other two forms run.  The chain is the same, bit for bit.
  * Paper: Sec. 3.1 (the schedule), Sec. 4.1 (scans of small lattices).
  * Errors: EINVAL (null argument, mode not 0-2).
@@ -258,18 +259,24 @@ int ising_batch_set_cluster(ising_batch_t b, int32_t mode);
 int ising_batch_cluster_size(ising_batch_t b, int32_t *cluster_size);
 
 /*
- * The workspace for random numbers drawn ahead (ising_init_ex, ising_init3d: sides 64 and
- * 128).  mode ISING_WORKSPACE_BESIDE (the default): taken by the first run that gains by it,
- * kept until the handle is freed.  All workspaces of the process together hold at most 4 GB, and
+ * The workspace for random numbers drawn ahead (ising_init_ex, ising_init3d for sides 64 and
+ * 128, ising_batch_set_cluster).  mode ISING_WORKSPACE_BESIDE (the default): taken by the first run that gains by it,
+ * kept until the handle or batch is freed.  All such workspaces of the process together hold at most 4 GB, and
  * one of more than 4 MB takes at most a 64th of the device memory then free; where it cannot be had, the sweeps
  * run without it and it is tried again after 1,024 more.  ISING_WORKSPACE_NONE: never, and one held is
  * given back at once (the call then synchronises; a graph captured from a run that used
- * it must not be replayed any more).  The chain is the same either way, bit for bit.
- * Paper: none (memory of the Sec. 3.1 sweep).  Errors: EINVAL (null handle, mode), ECUDA.
+ * it must not be replayed any more).  ISING_WORKSPACE_ARENA (batches): in what the lattices leave
+ * of the batch's arena, so that arena_bytes bounds both; it gives way when a lattice needs the
+ * room, shrinks with what is left (4.25 or 2.25 bytes a site) and does not count in
+ * ising_batch_usage.  The chain is the same in every mode, bit for bit.
+ * Paper: none (memory of the Sec. 3.1 sweep).  Errors: EINVAL (null handle or batch, mode),
+ * ECUDA.
  */
 #define ISING_WORKSPACE_NONE 0
 #define ISING_WORKSPACE_BESIDE 1
+#define ISING_WORKSPACE_ARENA 2
 int ising_set_workspace(ising_t h, int32_t mode);
+int ising_batch_set_workspace(ising_batch_t b, int32_t mode);
 
 /*
  * What the last run with n > 0 sweeps was (ising_sweep; ising_batch_run): *form, the kernels

@@ -548,6 +548,7 @@ struct Workspace {
     }
 };
 std::atomic<int64_t> Workspace::held{0};
+constexpr int64_t kAheadRetry = 1024;  // sweeps after which one that could not be had is tried again
 
 // A handle's or batch's share in the report blocks (report_block.h).
 struct ReadbackUser {
@@ -588,6 +589,11 @@ struct ising_s {
     const void* cubic_fixed[2] = {nullptr, nullptr};  // 3D: the colours' compiled instances
 };
 
+// Sweeps in all from which a batch takes a workspace beside its arena, whose allocation costs about
+// 0.1 ms (us for the first run of a new batch, with it / without: 16 sweeps of 8 x 1,024 180 / 159,
+// of 48 x 1,024 496 / 422; 32 sweeps 232 / 300 and 813 / 821).
+constexpr int64_t kAheadMinBatchSweeps = 32;
+
 struct ising_batch_s {
     ReadbackUser readback;
     LastRun last;
@@ -605,14 +611,16 @@ struct ising_batch_s {
     bool growable = false;
     int cluster_mode = ISING_CLUSTER_AUTO;  // ising_batch_set_cluster
     // the sweep with its random numbers drawn ahead (update_ahead): whether it is chosen, its
-    // launch parameters, its workspace (and those it has outgrown, still in use by earlier
-    // launches), and whether its tables follow the slots
-    bool ahead_wanted = false, ahead_refused = false, ahead_tables = false;
+    // launch parameters, its workspace (ising_batch_set_workspace), and whether its tables
+    // follow the slots
+    bool ahead_wanted = false, ahead_tables = false, ahead_configured = false;
     AheadBatch ahead{};
-    int64_t ahead_steps = 0, ahead_asked = 0, ahead_sites = 0;
-    char* ahead_ws = nullptr;
-    int64_t ahead_ws_bytes = 0;
-    std::vector<void*> ahead_outgrown;
+    int ahead_chunk = 0;        // the longest that the sides allow; ahead.chunk: what the memory does
+    int64_t ahead_steps = 0, ahead_sites = 0, ahead_words = 0;
+    int64_t ahead_asked = 0, ahead_from = kAheadMinBatchSweeps;  // sweeps asked for; those from which the workspace is taken
+    int32_t workspace_mode = ISING_WORKSPACE_BESIDE;
+    Workspace ahead_ws;
+    int64_t ahead_off = 0, ahead_bytes = 0;  // its place in the arena (bytes = 0: none)
     int capacity = 0;
     int64_t max_L = 0;
     cudaStream_t stream = nullptr;
@@ -653,12 +661,6 @@ int ensure_hist(ising_t h, int64_t need)
 
 uint32_t thr32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : (uint32_t)T; }
 uint32_t all32(uint64_t T) { return T >= 4294967296ull ? 0xFFFFFFFFu : 0u; }
-
-cudaError_t malloc_relaxed(char** p, size_t bytes)
-{
-    RelaxedCapture relaxed;
-    return cudaMalloc(p, bytes);
-}
 
 // Sweeps in all from which a run takes the workspace: 16; of lattices that the resident kernel
 // sweeps, 96 (L = 64), 64 (128) and 32 (192).  It costs about 70 us, the other kernel's time for that
@@ -703,7 +705,6 @@ int setup_ahead(ising_t h)
 // that needs it once the handle has been asked for ahead_min_sweeps in all.  Before that, where
 // it cannot be had (tried again after kAheadRetry more sweeps) and on a stream that is being
 // captured, the resident or the tiled kernel runs; the chain is the same.
-constexpr int64_t kAheadRetry = 1024;
 bool ahead_ready(ising_t h, int64_t n)
 {
     const AheadPlan& p = h->ahead_plan;
@@ -1624,7 +1625,7 @@ int update_cluster(ising_batch_t b)
 //    32 uneven lattices of 2.1e7 sites 21.4 us, 9.5 drawn ahead); they cross at 1.2e8 sites;
 //  - cluster-resident: 3,000 + 1,420 for each word a thread holds of a plane (64 x 1,024: 16
 //    words, 25.7 us; 8 x 1,024: 8.7, drawn ahead 3.7; 256 x 128: 4.9 and 2.6).
-constexpr int64_t kAheadMaxBatchSites = 130000000;  // a workspace of 0.6 GB
+constexpr int64_t kAheadMaxBatchSites = 130000000;  // a workspace of 1.07 GB
 void update_ahead(ising_batch_t b)
 {
     b->ahead_wanted = false;
@@ -1649,18 +1650,17 @@ void update_ahead(ising_batch_t b)
     if (drawn_ahead >= other) return;
     b->ahead_wanted = true;
     b->ahead_sites = sites;
-    b->ahead.chunk = ahead_batch_chunk(longest);
+    b->ahead_words = sites / 64;
+    b->ahead_chunk = ahead_batch_chunk(longest);
     // tall tiles once a launch has work for every SM (us a sweep, low / tall tiles: 8 x 256
     // 0.75 / 1.08; 32 x 256 1.53 / 1.23; 16 x 512 2.40 / 2.36; 64 x 1,024 32.2 / 29.0)
     b->ahead.dense = S >= 2e6;
 }
 
 // Whether a run of n sweeps goes that way: the workspace and the tables are made ready by the
-// first run that needs them, once the batch has been asked for 32 sweeps in all (us for the first
-// run of a new batch, with the workspace's allocation / without: 16 sweeps of 8 x 1,024 180 / 159, of
-// 48 x 1,024 496 / 422; 32 sweeps 232 / 300 and 813 / 821).  Before that,
-// where memory is short and on a stream that is being captured: the tiled or the
-// cluster-resident kernel, as otherwise (the launches here carry the batch's tables by value, so
+// first run that needs them, once the batch has been asked for kAheadMinBatchSweeps in all (at once
+// where the workspace lies in the arena).  Before that, where memory is short and on a stream
+// that is being captured: the tiled or the cluster-resident kernel, as otherwise (the launches here carry the batch's tables by value, so
 // a graph of them would not follow a batch that changes between its replays).
 //
 // Runs of up to four sweeps have a launch that draws with nothing to update and one that updates
@@ -1676,13 +1676,75 @@ bool ahead_run_too_short(int64_t sites, int64_t n)
     return n <= 4 && sites >= kFrom[n];
 }
 
-constexpr int64_t kAheadMinBatchSweeps = 32;
+// A batch's workspace: tickets and tables, two mask buffers, two copies of the planes.  8.25 bytes a
+// site with chunks of 16 sweeps (sides up to 2,048), 4.25 with 8.
+struct AheadLayout {
+    int64_t tables, masks, bytes;
+    AheadLayout(int64_t words, int chunk)
+        : tables(256 + (3 * ((int64_t)ahead_batch_max_count() + 1) * 4 + 255) / 256 * 256),
+          masks((words * 2 * chunk * (int64_t)sizeof(uint2) + 255) / 256 * 256),
+          bytes(tables + 2 * masks + words * 16)
+    {
+    }
+};
+
+// Gives the workspace's place in the arena up (its next user comes later on the same stream).
+void ahead_leave_arena(ising_batch_t b)
+{
+    if (!b->ahead_bytes) return;
+    b->arena.release(b->ahead_off, b->ahead_bytes);
+    b->ahead_bytes = 0;
+    b->ahead_tables = false;
+}
+
+// What the lattices hold of the arena.
+int64_t arena_lattice_bytes(ising_batch_t b) { return b->arena.used - FreeList::round_up(b->ahead_bytes); }
+
+// A place for the workspace, and the chunk that fits it: the longest, or a half or a quarter where
+// memory is short (at least 4 sweeps a launch).  Null where none can be had.
+char* ahead_place(ising_batch_t b)
+{
+    const int least = std::min(b->ahead_chunk, 4);
+    auto bytes_of = [&](int chunk) { return AheadLayout(b->ahead_words, chunk).bytes; };
+    int& chunk = b->ahead.chunk;
+    if (b->workspace_mode == ISING_WORKSPACE_ARENA) {
+        ahead_leave_arena(b);
+        for (chunk = b->ahead_chunk; chunk >= least; chunk /= 2) {
+            const int64_t off = b->arena.alloc_top(bytes_of(chunk));
+            if (off < 0) continue;
+            b->ahead_off = off;
+            b->ahead_bytes = bytes_of(chunk);
+            return b->arena.base + off;
+        }
+        return nullptr;
+    }
+    Workspace& ws = b->ahead_ws;
+    chunk = b->ahead_chunk;
+    if (bytes_of(chunk) <= ws.bytes) return ws.p;
+    if (chunk / 2 >= least && bytes_of(chunk / 2) <= ws.bytes) {
+        chunk /= 2;
+        return ws.p;
+    }
+    // an outgrown one is given back first; half as much again for lattices yet to come
+    const bool outgrown = ws.p != nullptr;
+    if (outgrown) {
+        RelaxedCapture relaxed;
+        if (cudaStreamSynchronize(b->stream) != cudaSuccess) return nullptr;
+        ws.give();
+        const int64_t most = AheadLayout(kAheadMaxBatchSites / 64, ahead_batch_chunk(64)).bytes;
+        if (ws.take(std::min(bytes_of(chunk) / 2 * 3, std::max(most, bytes_of(chunk))))) return ws.p;
+    }
+    for (; chunk >= least; chunk /= 2)
+        if (ws.take(bytes_of(chunk))) return ws.p;
+    return nullptr;
+}
+
 int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
 {
     *ready = false;
-    b->ahead_asked = std::min<int64_t>(b->ahead_asked + n, kAheadMinBatchSweeps);
-    if (!b->ahead_wanted || b->ahead_refused || b->ahead_asked < kAheadMinBatchSweeps || ahead_run_too_short(b->ahead_sites, n))
-        return ISING_OK;
+    b->ahead_asked += n;
+    if (!b->ahead_wanted || b->workspace_mode == ISING_WORKSPACE_NONE || ahead_run_too_short(b->ahead_sites, n)) return ISING_OK;
+    if (b->workspace_mode == ISING_WORKSPACE_BESIDE && b->ahead_asked < b->ahead_from) return ISING_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(b->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
@@ -1693,6 +1755,15 @@ int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
         return ISING_OK;
     }
     AheadBatch& a = b->ahead;
+    char* const ws = ahead_place(b);
+    if (!ws) {
+        if (b->workspace_mode == ISING_WORKSPACE_BESIDE) b->ahead_from = b->ahead_asked + kAheadRetry;
+        return ISING_OK;
+    }
+    const AheadLayout lay(b->ahead_words, a.chunk);
+    if (!b->ahead_configured) CK(ahead_batch_configure());
+    b->ahead_configured = true;
+    CK(cudaMemsetAsync(ws, 0, 256, b->stream));
     std::vector<int32_t> t(3 * ((size_t)b->count + 1), 0);
     int32_t *tiles = t.data(), *steps = tiles + b->count + 1, *words = steps + b->count + 1;
     for (int k = 0; k < b->count; ++k) {
@@ -1701,33 +1772,12 @@ int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
         steps[k + 1] = steps[k] + (s.used ? ahead_batch_steps(s.L) : 0);
         words[k + 1] = words[k] + (s.used ? (int32_t)(s.L * (s.L / 64)) : 0);
     }
-    const int64_t W = words[b->count], table_bytes = 256 + (3 * ((int64_t)ahead_batch_max_count() + 1) * 4 + 255) / 256 * 256;
-    const int64_t mask_bytes = (W * 2 * a.chunk * (int64_t)sizeof(uint2) + 255) / 256 * 256;
-    const int64_t need = table_bytes + 2 * mask_bytes + W * 16;
-    if (need > b->ahead_ws_bytes) {
-        CK(ahead_batch_configure());
-        // half as much again for lattices yet to come; the outgrown workspace stays until the
-        // batch is freed, as earlier launches may still use it (all of them together are at
-        // most twice the last one)
-        char* ws = nullptr;
-        const int64_t bytes = b->ahead_ws ? need + need / 2 : need;
-        if (malloc_relaxed(&ws, (size_t)bytes) != cudaSuccess) {
-            cudaGetLastError();
-            b->ahead_refused = true;
-            return ISING_OK;
-        }
-        if (b->ahead_ws) b->ahead_outgrown.push_back(b->ahead_ws);
-        b->ahead_ws = ws;
-        b->ahead_ws_bytes = bytes;
-        CK(cudaMemsetAsync(ws, 0, 256, b->stream));
-    }
-    char* ws = b->ahead_ws;
     a.desc = b->eng.d_desc;
     a.ticket = reinterpret_cast<int*>(ws);
     a.tables = reinterpret_cast<const int32_t*>(ws + 256);
-    a.masks[0] = reinterpret_cast<uint2*>(ws + table_bytes);
-    a.masks[1] = reinterpret_cast<uint2*>(ws + table_bytes + mask_bytes);
-    a.copy = reinterpret_cast<uint32_t*>(ws + table_bytes + 2 * mask_bytes);
+    a.masks[0] = reinterpret_cast<uint2*>(ws + lay.tables);
+    a.masks[1] = reinterpret_cast<uint2*>(ws + lay.tables + lay.masks);
+    a.copy = reinterpret_cast<uint32_t*>(ws + lay.tables + 2 * lay.masks);
     a.status = b->eng.d_status;
     a.count = b->count;
     a.tiles = tiles[b->count];
@@ -1958,7 +2008,12 @@ int ising_batch_add_tiled(ising_batch_t b, int64_t L, double beta, uint64_t seed
     const int64_t bytes = plane_bytes + (b->growable ? 0 : 16 * sweeps);
     int64_t* own_hist = nullptr;
     if (b->growable) CK(cudaMalloc(&own_hist, 16 * (size_t)sweeps));
-    const int64_t off = b->arena.alloc(bytes);
+    int64_t off = b->arena.alloc(bytes);
+    if (off < 0 && b->ahead_bytes) {
+        // a workspace in the arena gives way to lattices
+        ahead_leave_arena(b);
+        off = b->arena.alloc(bytes);
+    }
     if (off < 0) {
         cudaFree(own_hist);
         return fail(ISING_ENOMEM, "arena full: %lld of %lld bytes used, need %lld", (long long)b->arena.used,
@@ -2085,6 +2140,22 @@ int ising_batch_set_cluster(ising_batch_t b, int32_t mode)
     return rc;
 }
 
+int ising_batch_set_workspace(ising_batch_t b, int32_t mode)
+{
+    if (!b) return fail(ISING_EINVAL, "null batch");
+    if (mode != ISING_WORKSPACE_NONE && mode != ISING_WORKSPACE_BESIDE && mode != ISING_WORKSPACE_ARENA)
+        return fail(ISING_EINVAL, "workspace mode %d is not 0, 1 or 2", mode);
+    if (mode == b->workspace_mode) return ISING_OK;
+    ahead_leave_arena(b);
+    if (b->ahead_ws.p) {
+        CK(cudaStreamSynchronize(b->stream));
+        b->ahead_ws.give();
+    }
+    b->ahead_tables = false;
+    b->workspace_mode = mode;
+    return ISING_OK;
+}
+
 int ising_batch_cluster_size(ising_batch_t b, int32_t* cluster_size)
 {
     if (!b || !cluster_size) return fail(ISING_EINVAL, "null argument");
@@ -2207,7 +2278,7 @@ int ising_batch_get_lattice(ising_batch_t b, int32_t idx, int8_t* out)
 int ising_batch_usage(ising_batch_t b, int64_t* arena_used, int32_t* slots_used)
 {
     if (!b) return fail(ISING_EINVAL, "null batch");
-    if (arena_used) *arena_used = b->arena.used;
+    if (arena_used) *arena_used = arena_lattice_bytes(b);
     if (slots_used) {
         int32_t n = 0;
         for (const auto& s : b->slots) n += s.used ? 1 : 0;
@@ -2229,8 +2300,7 @@ int ising_batch_free(ising_batch_t b)
     b->eng.destroy();
     b->arena.destroy();
     for (auto& s : b->slots) cudaFree(s.own_hist);
-    cudaFree(b->ahead_ws);
-    for (void* p : b->ahead_outgrown) cudaFree(p);
+    b->ahead_ws.give();
     cudaFree(b->d_me);
     cudaFree(b->d_read);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);

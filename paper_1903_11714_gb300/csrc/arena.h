@@ -41,7 +41,23 @@ struct FreeList {
         }
         return -1;
     }
-    // returns a block that alloc gave out (same offset and byte count)
+    // as alloc, but from the end of the last free block that fits: for a block that is given up
+    // again when the others need the room
+    int64_t alloc_top(int64_t bytes)
+    {
+        bytes = round_up(bytes);
+        for (auto it = free_.rbegin(); it != free_.rend(); ++it) {
+            if (it->second >= bytes) {
+                const int64_t off = it->first + it->second - bytes;
+                it->second -= bytes;
+                if (it->second == 0) free_.erase(std::next(it).base());
+                used += bytes;
+                return off;
+            }
+        }
+        return -1;
+    }
+    // returns a block that alloc or alloc_top gave out (same offset and byte count)
     void release(int64_t off, int64_t bytes)
     {
         bytes = round_up(bytes);

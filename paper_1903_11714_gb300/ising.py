@@ -70,6 +70,7 @@ _SIGS = {
     "ising_batch_cluster_size": (ctypes.c_int, [_vp, _P(_i32)]),
     "ising_batch_last_run": (ctypes.c_int, [_vp, _P(_i32), _P(_i64)]),
     "ising_set_workspace": (ctypes.c_int, [_vp, _i32]),
+    "ising_batch_set_workspace": (ctypes.c_int, [_vp, _i32]),
     "ising_last_run": (ctypes.c_int, [_vp, _P(_i32), _P(_i64)]),
     "ising_batch_observables_ex": (ctypes.c_int, [_vp, _i32, _P(_i64), _P(_i64), _P(_i64)]),
     "ising_batch_history": (ctypes.c_int, [_vp, _i32, _i64, _i64, _P(_i64), _P(_i64)]),
@@ -224,7 +225,7 @@ def ising_batch_observables(b: int, idx: int) -> tuple[int, int]:
 
 SPECIALIZE_OFF, SPECIALIZE_AUTO, SPECIALIZE_ALWAYS = 0, 1, 2
 CLUSTER_OFF, CLUSTER_AUTO, CLUSTER_ALWAYS = 0, 1, 2
-WORKSPACE_NONE, WORKSPACE_BESIDE = 0, 1
+WORKSPACE_NONE, WORKSPACE_BESIDE, WORKSPACE_ARENA = 0, 1, 2
 RUN_NONE, RUN_TILED, RUN_AHEAD, RUN_CLUSTER, RUN_BYTES, RUN_CUBIC, RUN_RESIDENT = range(7)
 
 
@@ -535,6 +536,11 @@ class Batch:
         c = ctypes.c_int32()
         _check(lib().ising_batch_cluster_size(self.b, ctypes.byref(c)))
         return c.value
+
+    def set_workspace(self, mode: int) -> None:
+        """WORKSPACE_BESIDE (default), _ARENA or _NONE: where the random numbers drawn ahead are kept
+        (beside the arena, in what the lattices leave of it, or not drawn ahead)."""
+        _check(lib().ising_batch_set_workspace(self.b, int(mode)))
 
     def gather(self, idx, out_ptr: int) -> None:
         """Enqueue (sweeps done, M, E) of slots idx into out_ptr (3 int64 each,

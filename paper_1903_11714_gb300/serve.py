@@ -4,9 +4,10 @@ Requests (L, beta, seed, sweeps) arrive over time.  A request is admitted as
 soon as a slot is free and its device-resident state (bit-packed planes, L^2/8
 bytes, plus 16 bytes of M/E history per sweep) fits in the HBM budget (the
 batch arena).  Every scheduling quantum enqueues q sweeps of all admitted
-lattices as one persistent launch per half-sweep (replayed from a CUDA graph
-captured once per quantum size), so requests that arrive while others run share
-the same launches.  A lattice stops at its own sweep count.
+lattices in common launches (one persistent launch per half-sweep, replayed from
+a CUDA graph captured once per quantum size, or, in what the lattices leave of the budget,
+chunks of sweeps with their random numbers drawn ahead), so requests that arrive while
+others run share the same launches.  A lattice stops at its own sweep count.
 
 The host never waits for the GPU between quanta: up to two quanta are in flight;
 a request is admitted (its start state and descriptor enqueued) while earlier
@@ -142,6 +143,8 @@ class Server:
             self.stream = stream
             self._bufs = [np.zeros(3 * self.slots, dtype=np.int64) for _ in range(self.IN_FLIGHT + 1)]
         self.batch = ising.Batch(self.slots, max_L, self.budget, threads, self.stream)
+        if device_events:
+            self.batch.set_workspace(ising.WORKSPACE_ARENA)  # random numbers drawn ahead stay within the budget
 
     @staticmethod
     def request_bytes(L: int, sweeps: int) -> int:
