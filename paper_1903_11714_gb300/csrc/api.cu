@@ -1701,30 +1701,35 @@ void ahead_leave_arena(ising_batch_t b)
 int64_t arena_lattice_bytes(ising_batch_t b) { return b->arena.used - FreeList::round_up(b->ahead_bytes); }
 
 // A place for the workspace, and the chunk that fits it: the longest, or a half or a quarter where
-// memory is short (at least 4 sweeps a launch).  Null where none can be had.
-char* ahead_place(ising_batch_t b)
+// memory is short (at least 4 sweeps a launch).  Null where none can be had; *fresh: not the one held.
+char* ahead_place(ising_batch_t b, bool* fresh)
 {
     const int least = std::min(b->ahead_chunk, 4);
     auto bytes_of = [&](int chunk) { return AheadLayout(b->ahead_words, chunk).bytes; };
     int& chunk = b->ahead.chunk;
+    chunk = b->ahead_chunk;
+    *fresh = false;
     if (b->workspace_mode == ISING_WORKSPACE_ARENA) {
+        if (bytes_of(chunk) <= b->ahead_bytes) return b->arena.base + b->ahead_off;
         ahead_leave_arena(b);
-        for (chunk = b->ahead_chunk; chunk >= least; chunk /= 2) {
-            const int64_t off = b->arena.alloc_top(bytes_of(chunk));
-            if (off < 0) continue;
-            b->ahead_off = off;
-            b->ahead_bytes = bytes_of(chunk);
-            return b->arena.base + off;
-        }
+        *fresh = true;
+        for (; chunk >= least; chunk /= 2)
+            for (const int64_t bytes : {bytes_of(chunk) / 2 * 3, bytes_of(chunk)}) {  // room for lattices yet to come
+                const int64_t off = b->arena.alloc_top(bytes);
+                if (off < 0) continue;
+                b->ahead_off = off;
+                b->ahead_bytes = bytes;
+                return b->arena.base + off;
+            }
         return nullptr;
     }
     Workspace& ws = b->ahead_ws;
-    chunk = b->ahead_chunk;
     if (bytes_of(chunk) <= ws.bytes) return ws.p;
     if (chunk / 2 >= least && bytes_of(chunk / 2) <= ws.bytes) {
         chunk /= 2;
         return ws.p;
     }
+    *fresh = true;
     // an outgrown one is given back first; half as much again for lattices yet to come
     const bool outgrown = ws.p != nullptr;
     if (outgrown) {
@@ -1755,7 +1760,8 @@ int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
         return ISING_OK;
     }
     AheadBatch& a = b->ahead;
-    char* const ws = ahead_place(b);
+    bool fresh = false;
+    char* const ws = ahead_place(b, &fresh);
     if (!ws) {
         if (b->workspace_mode == ISING_WORKSPACE_BESIDE) b->ahead_from = b->ahead_asked + kAheadRetry;
         return ISING_OK;
@@ -1763,7 +1769,7 @@ int ahead_ready(ising_batch_t b, int64_t n, bool* ready)
     const AheadLayout lay(b->ahead_words, a.chunk);
     if (!b->ahead_configured) CK(ahead_batch_configure());
     b->ahead_configured = true;
-    CK(cudaMemsetAsync(ws, 0, 256, b->stream));
+    if (fresh) CK(cudaMemsetAsync(ws, 0, 256, b->stream));
     std::vector<int32_t> t(3 * ((size_t)b->count + 1), 0);
     int32_t *tiles = t.data(), *steps = tiles + b->count + 1, *words = steps + b->count + 1;
     for (int k = 0; k < b->count; ++k) {
