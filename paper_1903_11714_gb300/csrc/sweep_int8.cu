@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 2) int8_half_sweep_seg64_kernel(cons
 // L % 64 != 0: a plane word is eight consecutive 8-byte chunks in row-major order (the lattice
 // has L / 8 chunks a row, each four target sites of either colour), which may lie in
 // several rows.  One thread per word: drawn once for its 32 sites instead of once for each of
-// its chunks (L = 1,000: 13.0 us a sweep, 14.4 before).
+// its chunks (us a sweep: L = 200 6.2, 8.7 before; 1,000 8.8, 14.4 before; 4,072 41, 94 before).
 __global__ void __launch_bounds__(kThreads) int8_half_sweep_chunk8_kernel(const Int8Sweep d)
 {
     const int64_t L = d.L;
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kThreads) int8_half_sweep_chunk8_kernel(const 
     const uint32_t thr[2] = {d.t2, d.t4};
     const uint32_t zero2 = (d.t2 == 0u && d.all2 == 0u) ? ~0u : 0u, zero4 = (d.t4 == 0u && d.all4 == 0u) ? ~0u : 0u;
     uint32_t negs = 0, anti = 0;
-    const int word = (int)(blockIdx.x * kThreads + threadIdx.x);
+    const int word = (int)(blockIdx.x * blockDim.x + threadIdx.x);
     const unsigned first = 8u * (unsigned)word;  // chunk, below 2^31
     int64_t i = first / (unsigned)G;
     int g = (int)(first - (unsigned)i * (unsigned)G);
@@ -415,8 +415,13 @@ cudaError_t launch_int8_half_sweep(int8_t* lat, int64_t L, uint64_t key, uint32_
         const int64_t grid = (segments / rows + kThreads - 1) / kThreads;
         return launch_following(int8_half_sweep_seg64_kernel, dim3((unsigned)grid), dim3(kThreads), 0, s, d, rows);
     }
-    const int64_t grid = (L * L / 64 + kThreads - 1) / kThreads;
-    return launch_following(int8_half_sweep_chunk8_kernel, dim3((unsigned)grid), dim3(kThreads), 0, s, d);
+    // small blocks, so that a small lattice's words lie on as many SMs as possible.  us a sweep with blocks of
+    // 32 / 64 / 128 / 256: L = 200: 6.1 / 6.2 / 6.7 / 9.0; 488: 6.4 / 6.6 / 7.1 / 9.2; 1,000: 8.3 / 8.8 / 9.7 / 13.0; 1,496:
+    // 14.2 / 14.0 / 13.8 / 13.9; 2,504: 23.1 / 20.4 / 19.9 / 20.3; 4,072: 43.0 / 41.0 / 40.7 / 42.6
+    const int64_t words = L * L / 64;
+    const int threads = words < 128ll * sm_count() ? 64 : 128;
+    return launch_following(int8_half_sweep_chunk8_kernel, dim3((unsigned)((words + threads - 1) / threads)), dim3(threads),
+                            0, s, d);
 }
 
 cudaError_t launch_int8_observe(const int8_t* lat, int64_t L, int64_t* ME, cudaStream_t s)

@@ -3,6 +3,7 @@ without a strip of their own still finish words of the warp's queue, and what th
 import numpy as np
 import pytest
 
+import oracle
 from paper_1903_11714_gb300 import build as libbuild
 from paper_1903_11714_gb300 import ising
 
@@ -29,3 +30,15 @@ def test_last_warp_counts(L, beta, start):
     (M, E, got), (m, e, ref) = out
     assert np.array_equal(got, ref)
     assert np.array_equal(M, m) and np.array_equal(E, e)
+
+
+# sides that are no multiple of 64: one word a thread, in blocks of 64 and, from 128 words an SM on, of 128
+# threads; whole blocks and a last one with a few words
+@pytest.mark.parametrize("L", [8, 88, 200, 488, 1080, 1096, 1112, 1128])
+def test_word_blocks(L):
+    lat = ising.Lattice(L, 0.42, L, ising.HOT, ising.INT8).sweep(12)
+    ref, M, E, _ = oracle.run(L, 0.42, L, oracle.HOT, 12)
+    m, e = lat.history(0, 12)
+    assert np.array_equal(m, M) and np.array_equal(e, E)
+    assert np.array_equal(lat.get_lattice(), ref)
+    lat.close()
